@@ -215,6 +215,21 @@ int lbm_set_block(lbm_t *h, int bx, int by);
 #define LBM_KERNEL_TMA 6
 int lbm_set_kernel(lbm_t *h, int variant);
 
+/* Two steps per launch (LBM_KERNEL_X2, periodic axes and halfway walls):
+ * calls of four or more steps may advance two steps per launch, the state
+ * between them kept in shared memory, in groups of four steps, so that the
+ * result is in the same buffer as after single steps. The other steps and
+ * steps that write rho and u take one launch each. Results are identical.
+ * After such a call the other buffer of the pair holds an earlier state, not
+ * always the one before the last step. LBM_FUSE_AUTO (default): for the
+ * lattices that it is faster for (FP32 from 400,000 nodes on, and short rows);
+ * LBM_FUSE_OFF: never; LBM_FUSE_ALWAYS: whenever the kernel and the walls
+ * allow it. Returns LBM_EINVAL for any other mode. */
+#define LBM_FUSE_AUTO 0
+#define LBM_FUSE_OFF 1
+#define LBM_FUSE_ALWAYS 2
+int lbm_set_fusion(lbm_t *h, int mode);
+
 /* How the one-node kernel applies bounce-back: LBM_WALLS_SELECT picks each
  * direction's load address (pulled neighbour or opposite direction at the
  * node) for every node, with no divergence; LBM_WALLS_BRANCH gathers as if
@@ -230,10 +245,10 @@ int lbm_set_kernel(lbm_t *h, int variant);
 int lbm_set_wall_mode(lbm_t *h, int mode);
 
 /* Multi-step calls (lbm_step, lbm_step_moments, lbm_run_host with n > 1)
- * replay CUDA graphs of `steps` consecutive launches instead of launching
- * each step: one graph per starting buffer, captured on first use on a
+ * replay CUDA graphs of `steps` consecutive steps instead of launching
+ * each: one graph per starting buffer, captured on first use on a
  * private stream and again after any change of the launch configuration
- * (bind, tau, lid, block, kernel, wall mode). Removes the per-launch gap that
+ * (bind, tau, lid, block, kernel, fusion, wall mode). Removes the per-launch gap that
  * dominates small (L2-resident) lattices. `steps` even in [2, 1024], or 0 for
  * plain launches only (default 32). While the bound stream is itself being
  * captured, plain launches are used. Results are identical either way. */
@@ -247,7 +262,8 @@ int lbm_set_pair_block(lbm_t *h, int bxp, int by);
 /* Launch-shape autotuner (no counterpart in the paper, which fixed its block
  * shape by hand, Sec. 6). Times every x-dominant block shape (32..256 threads
  * along x, at most the rounded-up row; 1..8 rows; 64..256 threads) of the
- * current kernel variant (the pair block for LBM_KERNEL_PAIR) over `steps`
+ * current kernel variant (the pair block for LBM_KERNEL_PAIR; one step per
+ * launch) over `steps`
  * calls of lbm_step after the same number untimed, with CUDA events on the
  * bound stream, and applies the fastest. This ADVANCES THE STATE by all the
  * steps it runs: tune before initialising the state you want.

@@ -54,6 +54,9 @@ LBM_KERNEL_BULK1 = 3
 LBM_KERNEL_X2 = 4
 LBM_KERNEL_X4 = 5
 LBM_KERNEL_TMA = 6
+LBM_FUSE_AUTO = 0
+LBM_FUSE_OFF = 1
+LBM_FUSE_ALWAYS = 2
 
 
 class LBMError(RuntimeError):
@@ -92,6 +95,7 @@ _SIGNATURES = {
     "lbm_set_kernel": [_vp, _i],
     "lbm_set_pair_block": [_vp, _i, _i],
     "lbm_set_wall_mode": [_vp, _i],
+    "lbm_set_fusion": [_vp, _i],
     "lbm_set_graph_steps": [_vp, _i],
     "lbm_autotune": [_vp, ctypes.c_char_p, _i, _vp, _vp, _vp],
     "lbm_current": [_vp, ctypes.POINTER(_vp), ctypes.POINTER(_vp)],

@@ -166,7 +166,7 @@ __device__ __forceinline__ T ldcg_pf(const T *p) {
 
 // ---- accessors ---------------------------------------------------------------
 // LBM_LD: plain load; LBM_LDV: volatile load; LBM_LDG: read-only
-// (non-coherent) path; LBM_LDCG: L2 only (both with the prefetch hint
+// (non-coherent) path; LBM_LDGN: the same without the hint; LBM_LDCG: L2 only (both with the prefetch hint
 // above where the type has one); LBM_ST: plain write-back store (*p = v);
 // LBM_ACC: plain *p += v; LBM_ATOMIC_ADD, LBM_ATOMIC_OR: atomicAdd,
 // atomicOr; LBM_VALID(p): whether the whole object at p may be read (for
@@ -216,6 +216,7 @@ __device__ __forceinline__ bool chk_valid(const T *p) {
 #define LBM_LDV(p) ::lbm::chk_ldv(p)
 #define LBM_LDG(p) ::lbm::chk_ldg(p)
 #define LBM_LDCG(p) ::lbm::chk_ldcg(p)
+#define LBM_LDGN(p) ::lbm::chk_ldg(p)
 #define LBM_ST(p, v) ::lbm::chk_st((p), (v))
 #define LBM_ACC(p, v) ::lbm::chk_acc((p), (v))
 #define LBM_ATOMIC_ADD(p, v) ::lbm::chk_atomic_add((p), (v))
@@ -226,6 +227,7 @@ __device__ __forceinline__ bool chk_valid(const T *p) {
 #define LBM_LDV(p) (*(const volatile decltype(+*(p)) *)(p))
 #define LBM_LDG(p) ::lbm::ldg_pf(p)
 #define LBM_LDCG(p) ::lbm::ldcg_pf(p)
+#define LBM_LDGN(p) __ldg(p)
 #define LBM_ST(p, v) ((void)(*(p) = (v)))
 #define LBM_ACC(p, v) ((void)(*(p) += (v)))
 #define LBM_ATOMIC_ADD(p, v) atomicAdd((p), (v))

@@ -66,6 +66,18 @@ cudaError_t launch_step(int storage, bool moments, const StepArgs &a, int bx,
 // threads (bxp pairs per block row, `by` rows).
 cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &a, int bxp, int by,
                            cudaStream_t s);
+// Two steps per launch (step2.cuh): tiles of w x h columns, ntx x nty of
+// them, the planes cut into `chunks` runs.
+struct Step2Plan {
+  int w, h, ntx, nty, chunks;
+  float us;  // modelled time of a pass
+};
+// Whether multi-step calls of this lattice are faster so.
+bool step2_wins(int storage, int nx, int ny, int nz);
+// Once per handle and device before its launches.
+cudaError_t prepare_step2(int storage, const StepArgs &a);
+Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms);
+cudaError_t launch_step2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s);
 cudaError_t launch_step_pair16(int storage, bool moments, const StepArgs &a, int bxp, int by,
                                cudaStream_t s);
 // Four x-adjacent nodes per thread (bxq groups of four per block row, `by`
@@ -232,8 +244,10 @@ struct lbm_lattice {
   bool bound;
   int bx, by;
   int kernel;    // LBM_KERNEL_NODE, LBM_KERNEL_PAIR or LBM_KERNEL_BULK*
+  int fuse;      // LBM_FUSE_AUTO / OFF / ALWAYS
   int wall_mode; // LBM_WALLS_AUTO / BRANCH / SELECT
   int sms;       // SM count of the bound device
+  lbm::Step2Plan plan2;  // tiles of the two-step kernel (w = 0: not made yet)
   int pbx, pby;  // block shape of the pair kernel (pairs along x, rows)
   int device;
   lbm::Scratch scr;

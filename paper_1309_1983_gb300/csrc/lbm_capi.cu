@@ -179,6 +179,36 @@ cudaError_t launch_one_step(const lbm_t *h, bool mom, const StepArgs &a) {
   return launch_one_step(h, mom, a, h->stream);
 }
 
+// Whether multi-step calls advance two steps per launch.
+bool fuses(const lbm_t *h) {
+  if (h->kernel != LBM_KERNEL_X2 || onsite(h) || h->fuse == LBM_FUSE_OFF) return false;
+  return h->fuse == LBM_FUSE_ALWAYS || lbm::step2_wins(h->storage, h->nx, h->ny, h->nz);
+}
+
+// The two-step kernel's tiles, made before the first launch that needs them.
+int ensure_plan2(lbm_t *h) {
+  if (h->plan2.w != 0 || !fuses(h)) return LBM_OK;
+  LBM_CUDA(lbm::prepare_step2(h->storage, make_args(h, nullptr, nullptr)), "two-step kernel setup");
+  h->plan2 = lbm::step2_plan(h->storage, h->nx, h->ny, h->nz, h->sms);
+  return LBM_OK;
+}
+
+// n steps from buffer c on stream s: whole groups of four as two launches of
+// two steps each (after a group the state is back in buffer c, as after four
+// single steps), the rest one launch per step. *c_end: the buffer that holds
+// the result, c after an even number of steps, else the other one.
+cudaError_t enqueue_steps(const lbm_t *h, int n, int c, cudaStream_t s, int *c_end) {
+  cudaError_t e = cudaSuccess;
+  if (fuses(h))
+    for (; n >= 4 && e == cudaSuccess; n -= 4)
+      for (int k = 0; k < 2 && e == cudaSuccess; ++k, c ^= 1)
+        e = lbm::launch_step2(h->storage, make_args(h, h->f[c], h->f[1 - c]), h->plan2, s);
+  for (; n > 0 && e == cudaSuccess; --n, c ^= 1)
+    e = launch_one_step(h, false, make_args(h, h->f[c], h->f[1 - c]), s);
+  *c_end = c;
+  return e;
+}
+
 void drop_graphs(lbm_t *h) {
   for (int p = 0; p < 2; ++p) {
     if (h->gexec[p]) cudaGraphExecDestroy(h->gexec[p]);
@@ -198,11 +228,8 @@ int step_graph(lbm_t *h, int p, cudaGraphExec_t *out) {
   if (!h->gcap)
     LBM_CUDA(cudaStreamCreateWithFlags(&h->gcap, cudaStreamNonBlocking), "stream create");
   LBM_CUDA(cudaStreamBeginCapture(h->gcap, cudaStreamCaptureModeThreadLocal), "graph capture");
-  cudaError_t e = cudaSuccess;
-  for (int k = 0; k < h->graph_steps && e == cudaSuccess; ++k) {
-    const int c = p ^ (k & 1);
-    e = launch_one_step(h, false, make_args(h, h->f[c], h->f[1 - c]), h->gcap);
-  }
+  int end = p;
+  cudaError_t e = enqueue_steps(h, h->graph_steps, p, h->gcap, &end);
   cudaGraph_t g = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(h->gcap, &g);
   if (e == cudaSuccess) e = e2;
@@ -257,6 +284,8 @@ void release_pipeline(lbm_t *h) {
 }
 
 int do_steps(lbm_t *h, int n, float *rho, float *u) {
+  int rc = ensure_plan2(h);
+  if (rc) return rc;
   // whole graphs first (an even number of steps each, so the current buffer
   // is unchanged), then plain launches; a step writing rho, u is always plain
   const int G = h->graph_steps;
@@ -265,24 +294,22 @@ int do_steps(lbm_t *h, int n, float *rho, float *u) {
     LBM_CUDA(cudaStreamIsCapturing(h->stream, &cs), "stream query");
     if (cs == cudaStreamCaptureStatusNone) {
       cudaGraphExec_t ge = nullptr;
-      int rc = step_graph(h, h->cur, &ge);
+      rc = step_graph(h, h->cur, &ge);
       if (rc) return rc;
       const int reps = (n - (rho ? 1 : 0)) / G;
       for (int r = 0; r < reps; ++r) LBM_CUDA(cudaGraphLaunch(ge, h->stream), "graph launch");
       n -= reps * G;
     }
   }
-  for (int k = 0; k < n; ++k) {
+  cudaError_t e = enqueue_steps(h, n - (rho ? 1 : 0), h->cur, h->stream, &h->cur);
+  if (e == cudaSuccess && rho) {
     StepArgs a = make_args(h, h->f[h->cur], h->f[1 - h->cur]);
-    const bool mom = (rho != nullptr) && (k == n - 1);
-    if (mom) {
-      a.rho = rho;
-      a.u = u;
-    }
-    cudaError_t e = launch_one_step(h, mom, a);
-    if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
-    h->cur ^= 1;
+    a.rho = rho;
+    a.u = u;
+    e = launch_one_step(h, true, a);
+    if (e == cudaSuccess) h->cur ^= 1;
   }
+  if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
   return LBM_OK;
 }
 
@@ -405,6 +432,7 @@ int lbm_create(int nx, int ny, int nz, float tau, uint32_t flags,
   // two nodes per thread: fewer instructions per node (decisive where the
   // one-node kernel is issue-bound, 16-bit storage; about 1% with FP32)
   h->kernel = LBM_KERNEL_X2;
+  h->fuse = LBM_FUSE_AUTO;
   h->wall_mode = LBM_WALLS_AUTO;
   h->pbx = 64;  // 64 pairs x 2 rows measured best for the two-node kernel
   h->pby = ny < 2 ? ny : 2;
@@ -472,6 +500,7 @@ int lbm_bind(lbm_t *h, void *f_a, void *f_b, const float *force, void *stream) {
   if (force && !aligned(force, 4)) return fail(LBM_EINVAL, "force misaligned");
   int rc = ensure_scratch(h);
   if (rc) return rc;
+  h->plan2 = lbm::Step2Plan{};
   h->f[0] = f_a;
   h->f[1] = f_b;
   h->cur = 0;
@@ -527,6 +556,14 @@ int lbm_set_kernel(lbm_t *h, int variant) {
   if (onsite(h) && variant != LBM_KERNEL_X2 && variant != LBM_KERNEL_NODE)
     return fail(LBM_EINVAL, "on-site walls run on LBM_KERNEL_X2 or LBM_KERNEL_NODE");
   h->kernel = variant;
+  h->config_version++;
+  return LBM_OK;
+}
+
+int lbm_set_fusion(lbm_t *h, int mode) {
+  if (!h) return fail(LBM_EINVAL, "NULL handle");
+  if (mode < LBM_FUSE_AUTO || mode > LBM_FUSE_ALWAYS) return fail(LBM_EINVAL, "bad mode");
+  h->fuse = mode;
   h->config_version++;
   return LBM_OK;
 }

@@ -1,0 +1,189 @@
+// lbm_step2.cu - two steps of one lattice per launch (step2.cuh), for
+// multi-step calls.
+//
+// A single step reads and writes every value once, and at 384^3 FP32 that is
+// all it waits for (46.6 GLUPS, 7.1 TB/s). Two steps per pass halve that
+// traffic; what bounds the pass then is the traffic between L2 and the SMs
+// (7 TB/s: a tile also reads its rim, 190 bytes per node and pass for 32 x 14
+// tiles against 152) and, at 86% of the DRAM rate of a copy, nearly DRAM.
+// Measured on GB300, MLUPS x 1e-3, one step per launch against two:
+//   periodic FP32   128^3 43.6 / 58.7   256^3 46.0 / 72.4   384^3 46.6 / 68.8
+//   cavity FP32     128^3 43.8 / 55.4   256^3 46.1 / 60.0   384^3 46.6 / 61.2
+//   cavity FP32     23 x 374 x 236 28.5 / 44.5   273 x 213 x 113 42.1 / 53.3
+//   periodic FP16   384^3 83.7 / 75.7   45 x 234 x 328 48.1 / 66.4
+// 16-bit storage moves half the bytes, so there the two collisions and the
+// conversions bound the pass.
+//
+// One block per SM of 9 + 7 warps at 128 registers. Tried and slower, 384^3
+// periodic FP32: all warps alternating between the two steps with a barrier
+// after each (48.6 without, 65.3 with the next plane's loads in flight over
+// the second step), 11 + 9 warps at 96 registers (59.9, spills), 7 + 5 at
+// 168 (61.2), two blocks of 5 + 3 warps, an L2 prefetch of the plane after
+// the next (60.3 against 65.3), and the 256-byte prefetch hint of the
+// single-step kernels (25.7: narrow tiles fetch their neighbours' values
+// several times over).
+#include "step2.cuh"
+
+#include <algorithm>
+
+#include "internal.h"
+
+namespace lbm {
+
+// Threads of the first step (two nodes each, so a tile with its rim has at
+// most kStep2Cap nodes) and of the second.
+constexpr int kFirst = 288, kSecond = 224;
+constexpr int kStep2Threads = kFirst + kSecond;
+constexpr int kStep2Cap = 2 * kFirst;
+
+template <int S>
+struct Step2Args {
+  Dom2<S> dom;
+  PairConsts consts;
+  float lidc[Q];
+  Step2Plan plan;
+};
+
+// One block per tile and chunk of planes; blocks of one chunk are neighbours
+// in the grid, so that neighbouring tiles walk the same planes at the same
+// time and find each other's rims in L2.
+template <int S, bool WALLS, bool FORCE>
+__global__ void __launch_bounds__(kStep2Threads, 1)
+    k_step2(const __grid_constant__ Step2Args<S> a) {
+  const Step2Plan &p = a.plan;
+  const Dom2<S> &D = a.dom;
+  using T = typename Store<S>::T;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T *ring = reinterpret_cast<T *>(smem_raw);
+  const int ntiles = p.ntx * p.nty;
+  const int chunk = (int)blockIdx.x / ntiles, tile = (int)blockIdx.x - chunk * ntiles;
+  const int ty = tile / p.ntx, tx = tile - ty * p.ntx;
+  const int x0 = tx * p.w, y0 = ty * p.h;
+  const int za = (int)((long long)D.nz * chunk / p.chunks);
+  const int zb = (int)((long long)D.nz * (chunk + 1) / p.chunks);
+  const int cw = min(p.w, D.nx - x0), ch = min(p.h, D.ny - y0);
+  const int t = threadIdx.x;
+  if (t < kFirst) {
+    // a tile away from the x and y walls takes the shorter form
+    const bool side = WALLS && (((D.walls & LBM_WALL_X) && (x0 <= 1 || x0 + cw >= D.nx - 1)) ||
+                                ((D.walls & LBM_WALL_Y) && (y0 <= 1 || y0 + ch >= D.ny - 1)));
+    if (side)
+      step2_first<S, WALLS ? 2 : 0, WALLS, FORCE, kStep2Cap>(ring, D, a.consts, a.lidc, x0, y0,
+                                                             cw, ch, za, zb, t);
+    else
+      step2_first<S, WALLS ? 1 : 0, WALLS, FORCE, kStep2Cap>(ring, D, a.consts, a.lidc, x0, y0,
+                                                             cw, ch, za, zb, t);
+  } else {
+    step2_second<S, WALLS, FORCE, kStep2Cap>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za, zb,
+                                             t - kFirst);
+  }
+}
+
+size_t step2_smem(int storage, bool walls) {
+  return (size_t)step2_ring_values(walls) * kStep2Cap * elem_bytes_of(storage);
+}
+
+// The tile and the number of chunks with the least modelled time. One plane
+// of a tile takes the time of its traffic between L2 and the SM: per
+// direction a row of the rim is read (with the sectors at its ends, about 8
+// values more), a row of the tile written. Measured on tiles from 8 x 54 to
+// 64 x 12 with all SMs busy: 45 to 48 KB per us and SM. A chunk walks 3
+// planes more than it writes; the last wave of blocks counts in full.
+Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms) {
+  Step2Plan best = {};
+  const int bytes = elem_bytes_of(storage);
+  for (int w8 = 8; w8 < nx + 8 && w8 <= kSecond; w8 += 8) {
+    const int w = w8 < nx ? w8 : nx;
+    const int rows = std::min(kFirst / (w + 2), kSecond / w + 1);  // of the rim, per thread
+    for (int h = std::min(2 * rows - 2, ny); h >= 1; --h) {
+      const int ntx = (nx + w - 1) / w, nty = (ny + h - 1) / h;
+      const double kb = 0.019 * bytes * ((h + 2.0) * (w + 2 + 32 / bytes) + (double)h * w);
+      const double plane_us = std::max(0.1 + kb / 48.0, 0.9);
+      const long long tiles = (long long)ntx * nty;
+      for (int k = 0; k <= 16; ++k) {  // chunks that fill k waves of blocks
+        const int c = k == 0 ? 1 : (int)std::min<long long>(nz, (long long)k * sms / tiles);
+        if (c < 1) continue;
+        const long long blocks = tiles * c;
+        const double waves = (double)((blocks + sms - 1) / sms);
+        const double us = 2.0 + waves * ((nz + c - 1) / c + 3) * plane_us;
+        if (best.w == 0 || us < best.us) best = {w, h, ntx, nty, c, (float)us};
+      }
+    }
+  }
+  return best;
+}
+
+template <int S, bool WALLS, bool FORCE>
+static cudaError_t launch2(const StepArgs &a, const Step2Plan &p, size_t smem, cudaStream_t s) {
+  if (p.w == 0)  // the plan's preparation: allow this much shared memory
+    return cudaFuncSetAttribute(k_step2<S, WALLS, FORCE>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  Step2Args<S> b;
+  for (int i = 0; i < Q; ++i) {
+    b.dom.fin[i] = static_cast<const typename Store<S>::T *>(a.fin) + (size_t)i * a.plane;
+    b.dom.fout[i] = static_cast<typename Store<S>::T *>(a.fout) + (size_t)i * a.plane;
+    b.lidc[i] = a.lidc[i];
+  }
+  b.dom.force = a.force;
+  b.dom.nx = a.nx;
+  b.dom.ny = a.ny;
+  b.dom.nz = a.nz;
+  b.dom.pitch = a.pitch;
+  b.dom.plane = a.plane;
+  b.dom.cells = a.cells;
+  b.dom.walls = a.walls;
+  b.dom.omega = a.omega;
+  b.dom.kf = a.kf;
+  b.consts = pair_consts(a.omega);
+  b.plan = p;
+  k_step2<S, WALLS, FORCE><<<p.ntx * p.nty * p.chunks, kStep2Threads, smem, s>>>(b);
+  return cudaGetLastError();
+}
+
+static cudaError_t dispatch2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s) {
+  const bool walls = a.walls != 0, force = a.force != nullptr;
+  const size_t smem = step2_smem(storage, walls);
+#define LBM_STEP2_CASE(S, W, F) \
+  if (storage == S && walls == W && force == F) return launch2<S, W, F>(a, p, smem, s);
+  LBM_STEP2_CASE(0, false, false)
+  LBM_STEP2_CASE(0, false, true)
+  LBM_STEP2_CASE(0, true, false)
+  LBM_STEP2_CASE(0, true, true)
+  LBM_STEP2_CASE(1, false, false)
+  LBM_STEP2_CASE(1, false, true)
+  LBM_STEP2_CASE(1, true, false)
+  LBM_STEP2_CASE(1, true, true)
+  LBM_STEP2_CASE(2, false, false)
+  LBM_STEP2_CASE(2, false, true)
+  LBM_STEP2_CASE(2, true, false)
+  LBM_STEP2_CASE(2, true, true)
+#undef LBM_STEP2_CASE
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t prepare_step2(int storage, const StepArgs &a) {
+  return dispatch2(storage, a, Step2Plan{}, nullptr);
+}
+
+cudaError_t launch_step2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s) {
+  LBM_CHECK_TABLE(s, LBM_STEP_RANGES(a, elem_bytes_of(storage)));
+  return dispatch2(storage, a, p, s);
+}
+
+// Where two steps per launch are faster than two launches of the two-node
+// kernel. FP32: from 400,000 nodes on, where the lattice outgrows L2
+// (measured cavity, two launches against one: 96^3 19.8 / 15.9 us a step,
+// 72^3 9.0 / 10.1, 101 x 67 x 45 7.0 / 8.9, 78 x 237 x 27 11.2 / 9.9). 16-bit
+// storage: only where the two-node kernel's 128-node blocks fit the rows
+// badly (FP16 cavity, 45 x 234 x 328 74.7 / 59.2, 86 x 194 x 115 39.3 / 35.4,
+// 193 x 160 x 129 67.2 / 71.4). Rows of up to 30 nodes leave three quarters
+// of its threads idle, and two steps per launch win from 60,000 nodes on
+// (24 x 200 x 24 5.7 / 4.7, 20 x 60 x 60 4.6 / 4.4).
+bool step2_wins(int storage, int nx, int ny, int nz) {
+  const double nodes = (double)nx * ny * nz;
+  if (nx <= 30) return nodes >= 6e4;
+  if (nodes < 4e5) return false;
+  return storage == kF32 || nx < 0.7 * 128 * ((nx + 127) / 128);
+}
+
+}  // namespace lbm

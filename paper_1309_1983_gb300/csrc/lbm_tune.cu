@@ -118,7 +118,10 @@ int lbm_autotune(lbm_t *h, const char *cache_path, int steps, int *bx_out, int *
     int rc = pair ? lbm_set_pair_block(h, c.first, c.second) : lbm_set_block(h, c.first, c.second);
     if (rc) return rc;
     float ms = 0.f;
+    const int fuse = h->fuse;
+    h->fuse = LBM_FUSE_OFF;  // the shape is that of the launches of one step
     rc = lbm::time_calls(h->stream, 1, [&]() { return lbm_step(h, steps); }, &ms);
+    h->fuse = fuse;
     if (rc) return rc;
     ms /= steps;
     if (!best_a || ms < best_ms) {

@@ -1,0 +1,390 @@
+// step2.cuh - two time steps of a tile in one pass over memory.
+//
+// A block owns a tile of w x h output columns and walks along z. Its first
+// warps compute the first step of one plane after the other, on the tile and
+// a rim of one node around it (pull gather from global memory, collision),
+// and keep the results in shared memory only; its other warps follow two
+// planes behind and compute the second step from there. One block barrier
+// per plane: between two barriers the first warps work on plane k while the
+// others work on plane k - 2, so loads, collisions and stores of both steps
+// overlap. The state after the first step never goes to memory: per two
+// steps a node costs one read and one write (2 x 76 bytes in FP32) instead
+// of two of each; the rim's first step is computed by the tiles on both sides.
+//
+// Rings in shared memory (values as stored, so 16-bit storage rounds after
+// the first step as the single-step kernels do). The second step of plane
+// k - 2 pulls e_z = +1 values from plane k - 3, e_z = 0 from k - 2 and
+// e_z = -1 from k - 1 while plane k is being written: four planes of the 5
+// e_z = +1 directions, three of the 9 e_z = 0 and two of the 5 e_z = -1 are
+// live (three with walls: see below).
+//
+// Walls (halfway bounce-back): both steps take the opposite direction's
+// value at the node itself where a pull would come from beyond a wall. The
+// second step reads it from the node's own plane, which for e_z = -1 keeps a
+// third plane alive. Warps without a wall node skip the selection.
+#pragma once
+
+#include "d3q19.cuh"
+#include "pair_math.cuh"
+#include "stream.cuh"
+
+namespace lbm {
+
+// Number of directions before i with the same e_z: i's place in its ring.
+__host__ __device__ constexpr int ring_rank(int i) {
+  int r = 0;
+  for (int j = 0; j < i; ++j) r += kEz[j] == kEz[i];
+  return r;
+}
+
+// Values of shared memory per node of a tile with its rim.
+__host__ __device__ constexpr int step2_ring_values(bool walls) {
+  return 4 * 5 + 3 * 9 + (walls ? 3 : 2) * 5;
+}
+
+// Store to shared memory in the storage type.
+template <int S>
+__device__ __forceinline__ void st_ring(typename Store<S>::T *p, float v) {
+  if constexpr (S == 0)
+    *p = v;
+  else if constexpr (S == 1)
+    *p = __float2half_rn(v);
+  else
+    *p = __float2bfloat16_rn(v);
+}
+
+// A pulled pair as loaded (16-bit values are converted when they are used:
+// converting at once would wait for the load).
+template <int S>
+struct RawPair {
+  typename Store<S>::T a, b;
+};
+template <int S>
+__device__ __forceinline__ P2 as_pair(const RawPair<S> &r) {
+  if constexpr (S == 0)
+    return pk(r.a, r.b);
+  else if constexpr (S == 1)
+    return pk(__half2float(r.a), __half2float(r.b));
+  else
+    return pk(__bfloat162float(r.a), __bfloat162float(r.b));
+}
+
+// One lattice of a two-step pass. The direction planes come as ready
+// pointers: in a kernel parameter they are constant-bank operands of the
+// address arithmetic, one instruction per access.
+template <int S>
+struct Dom2 {
+  using T = typename Store<S>::T;
+  const T *fin[Q];
+  T *fout[Q];
+  const float *force;  // dense [3][cells] or nullptr
+  int nx, ny, nz, pitch;
+  uint32_t plane, cells, walls;
+  float omega, kf;
+};
+
+// Walled faces a node touches.
+enum : uint32_t { kX0 = 1, kX1 = 2, kY0 = 4, kY1 = 8, kZ0 = 16, kZ1 = 32 };
+
+// In-plane part of a node of the first step: its place in the tile's ring
+// arrays and the wrapped neighbour offsets.
+struct Rim {
+  uint32_t yo[3], xo[3];  // (plus, same, minus) neighbour per axis
+  int pos;                // place in a ring plane
+  uint32_t fc;            // dense node of its force in an xy plane
+  uint32_t faces;         // walled x and y faces
+  bool live;              // the node exists (not beyond a wall)
+};
+
+template <bool WALLS>
+__device__ __forceinline__ Rim rim_node(int idx, int n, int lx_n, int x0, int y0, int cw, int ch,
+                                        int nx, int ny, int pitch, uint32_t walls) {
+  Rim r;
+  const int k = idx < n ? idx : n - 1;
+  const int ly = k / lx_n, lx = k - ly * lx_n;
+  r.pos = k;
+  r.live = idx < n;
+  int gx = x0 + lx - 1, gy = y0 + ly - 1;
+  r.faces = 0;
+  if (WALLS && (walls & LBM_WALL_X)) {
+    r.live &= gx >= 0 && gx < nx;
+    gx = min(max(gx, 0), nx - 1);
+    r.faces |= (gx == 0 ? kX0 : 0u) | (gx == nx - 1 ? kX1 : 0u);
+  } else {
+    gx = gx < 0 ? gx + nx : gx >= nx ? gx - nx : gx;
+  }
+  if (WALLS && (walls & LBM_WALL_Y)) {
+    r.live &= gy >= 0 && gy < ny;
+    gy = min(max(gy, 0), ny - 1);
+    r.faces |= (gy == 0 ? kY0 : 0u) | (gy == ny - 1 ? kY1 : 0u);
+  } else {
+    gy = gy < 0 ? gy + ny : gy >= ny ? gy - ny : gy;
+  }
+  if (!r.live) r.faces = 0;
+  r.fc = (uint32_t)gy * nx + gx;
+  const int xm = gx == 0 ? nx - 1 : gx - 1, xp = gx == nx - 1 ? 0 : gx + 1;
+  const int ym = gy == 0 ? ny - 1 : gy - 1, yp = gy == ny - 1 ? 0 : gy + 1;
+  r.xo[0] = (uint32_t)xp;
+  r.xo[1] = (uint32_t)gx;
+  r.xo[2] = (uint32_t)xm;
+  r.yo[0] = (uint32_t)yp * pitch;
+  r.yo[1] = (uint32_t)gy * pitch;
+  r.yo[2] = (uint32_t)ym * pitch;
+  return r;
+}
+
+// The faces beyond which direction i is pulled.
+__host__ __device__ constexpr uint32_t beyond_xy(int i) {
+  return (kEx[i] == 1 ? kX0 : kEx[i] == -1 ? kX1 : 0u) |
+         (kEy[i] == 1 ? kY0 : kEy[i] == -1 ? kY1 : 0u);
+}
+__host__ __device__ constexpr uint32_t beyond_z(int i) {
+  return kEz[i] == 1 ? kZ0 : kEz[i] == -1 ? kZ1 : 0u;
+}
+
+// f(i) for the directions i pulled from beyond each face in `faces` (a
+// direction beyond two of them is visited twice).
+// `any`: the faces some node of the warp touches, so that a warp branches past
+// the others instead of issuing their instructions for no thread.
+template <class F>
+__device__ __forceinline__ void for_bounces(uint32_t faces, uint32_t any, F &&f) {
+  auto face = [&](auto Axis, auto Sgn) {
+    static_for<1, Q>([&](auto I) {
+      constexpr int i = decltype(I)::value, axis = decltype(Axis)::value;
+      constexpr int ex = kEx[i], ey = kEy[i], ez = kEz[i];
+      constexpr int e = axis == 0 ? ex : axis == 1 ? ey : ez;
+      if constexpr (e == decltype(Sgn)::value) f(I);
+    });
+  };
+  using std::integral_constant;
+  const integral_constant<int, 0> x;
+  const integral_constant<int, 1> y;
+  const integral_constant<int, 2> z;
+  const integral_constant<int, 1> low;
+  const integral_constant<int, -1> high;
+  if (any & kX0)
+    if (faces & kX0) face(x, low);
+  if (any & kX1)
+    if (faces & kX1) face(x, high);
+  if (any & kY0)
+    if (faces & kY0) face(y, low);
+  if (any & kY1)
+    if (faces & kY1) face(y, high);
+  if (any & kZ0)
+    if (faces & kZ0) face(z, low);
+  if (any & kZ1)
+    if (faces & kZ1) face(z, high);
+}
+
+// Where the values of direction i of a plane are kept: ring arrays of CAP
+// values each, per class of e_z `slots` planes of them.
+template <bool WALLS, int CAP>
+struct Ring {
+  static constexpr int kPlus = 0, kZero = 4 * 5 * CAP, kMinus = kZero + 3 * 9 * CAP;
+  static constexpr int kMinusSlots = WALLS ? 3 : 2;
+  // First value of direction i in a plane whose slots are given per class.
+  template <int i>
+  static __device__ __forceinline__ int at(int plus, int zero, int minus) {
+    constexpr int ez = kEz[i];
+    constexpr int r = ring_rank(i) * CAP;
+    if constexpr (ez == 1) return kPlus + plus * (5 * CAP) + r;
+    if constexpr (ez == 0) return kZero + zero * (9 * CAP) + r;
+    return kMinus + minus * (5 * CAP) + r;
+  }
+};
+
+// First step of planes za - 1 .. zb on the tile and its rim (the block's
+// first warps; t: thread among them). FACES: the walls that the tile may
+// touch: 0 none, 1 z faces, 2 any.
+template <int S, int FACES, bool WALLS, bool FORCE, int CAP>
+__device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ ring,
+                                            const Dom2<S> &D, const PairConsts &C,
+                                            const float (&lidc)[Q], int x0, int y0, int cw,
+                                            int ch, int za, int zb, int t) {
+  using T = typename Store<S>::T;
+  using R = Ring<WALLS, CAP>;
+  const int lx_n = cw + 2;
+  // the two nodes of a thread lie in the same column, half the rows apart, so
+  // that both touch an x wall or neither does
+  const int n1 = lx_n * (ch + 2), half1 = lx_n * ((ch + 3) >> 1);
+  const Rim A = rim_node<WALLS>(t, n1, lx_n, x0, y0, cw, ch, D.nx, D.ny, D.pitch, D.walls);
+  const Rim B = rim_node<WALLS>(t + half1, n1, lx_n, x0, y0, cw, ch, D.nx, D.ny, D.pitch, D.walls);
+  const uint32_t row = (uint32_t)D.ny * D.pitch;
+  const uint32_t drow = (uint32_t)D.ny * D.nx;
+  const bool wz = WALLS && (D.walls & LBM_WALL_Z);
+  const int planes = zb - za + 2;
+
+  // Pull gather of plane za - 1 + k for the thread's two nodes. Straight-line
+  // code: a branch here (or a later repair of the wall nodes' values) makes
+  // the compiler wait for the loads it should leave in flight.
+  auto pull = [&](int k, RawPair<S> (&d)[Q]) {
+    const int zr = za - 1 + k;
+    if (t >= half1 || (wz && (zr < 0 || zr >= D.nz))) return;
+    const int z = zr < 0 ? zr + D.nz : zr >= D.nz ? zr - D.nz : zr;
+    const uint32_t zo[3] = {(uint32_t)(z == D.nz - 1 ? 0 : z + 1) * row, (uint32_t)z * row,
+                            (uint32_t)(z == 0 ? D.nz - 1 : z - 1) * row};
+    const uint32_t zf = wz ? (z == 0 ? kZ0 : 0u) | (z == D.nz - 1 ? kZ1 : 0u) : 0u;
+    const uint32_t na = zo[1] + A.yo[1] + A.xo[1], nb = zo[1] + B.yo[1] + B.xo[1];
+    const uint32_t oa = na + D.plane, ob = nb + D.plane;
+    static_for<0, Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      constexpr int jx = 1 + kEx[i], jy = 1 + kEy[i], jz = 1 + kEz[i];
+      constexpr uint32_t mz = beyond_z(i), mxy = beyond_xy(i);
+      const uint32_t fa = zo[jz] + A.yo[jy] + A.xo[jx], fb = zo[jz] + B.yo[jy] + B.xo[jx];
+      if constexpr (FACES == 2 && (mz | mxy) != 0) {
+        // opposite directions are neighbours (odd, even): both offsets count
+        // from the odd one's plane, so a 32-bit selection picks the source
+        constexpr bool even = i % 2 == 0;
+        const T *base = D.fin[even ? i - 1 : i];
+        const bool ba = ((A.faces | zf) & (mz | mxy)) != 0;
+        const bool bb = ((B.faces | zf) & (mz | mxy)) != 0;
+        d[i].a = LBM_LDGN(base + (even ? (ba ? na : fa + D.plane) : (ba ? oa : fa)));
+        d[i].b = LBM_LDGN(base + (even ? (bb ? nb : fb + D.plane) : (bb ? ob : fb)));
+      } else if constexpr (FACES == 1 && mz != 0) {
+        const bool bz = (zf & mz) != 0;  // the same for all threads
+        const T *base = bz ? D.fin[kOpp_v<i>] : D.fin[i];
+        d[i].a = LBM_LDGN(base + (bz ? na : fa));
+        d[i].b = LBM_LDGN(base + (bz ? nb : fb));
+      } else {
+        d[i].a = LBM_LDGN(D.fin[i] + fa);
+        d[i].b = LBM_LDGN(D.fin[i] + fb);
+      }
+    });
+  };
+
+  RawPair<S> next[Q] = {};  // the next plane's pulled values, in flight meanwhile
+  pull(0, next);
+  int sp = 0, sz = 0, sm = 0;  // k modulo the number of slots, per class
+  for (int k = 0; k < planes; ++k) {
+    const int zr = za - 1 + k;
+    const int z = zr < 0 ? zr + D.nz : zr >= D.nz ? zr - D.nz : zr;
+    const bool exists = t < half1 && (!wz || (zr >= 0 && zr < D.nz));
+    const bool top = FACES != 0 && wz && z == D.nz - 1;
+    P2 d[Q];
+    static_for<0, Q>([&](auto I) {
+      constexpr int i = decltype(I)::value;
+      d[i] = as_pair<S>(next[i]);
+      if constexpr (FACES != 0 && kEz[i] == -1) d[i] = d[i] + pk(top ? lidc[i] : 0.0f);
+    });
+    if (k + 1 < planes) pull(k + 1, next);
+    if (exists) {
+      P2 rho, ux, uy, uz;
+      if constexpr (FORCE) {
+        const uint32_t ca = (uint32_t)z * drow + A.fc;
+        const uint32_t cb = (uint32_t)z * drow + B.fc;
+        collide_pair_force(d, D.omega, D.kf, D.force, D.cells, ca, cb, rho, ux, uy, uz);
+      } else {
+        collide_pair(d, C, rho, ux, uy, uz);
+      }
+      static_for<0, Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        T *p = ring + R::template at<i>(sp, sz, sm);
+        const float2 v = unpk(d[i]);
+        if (A.live) st_ring<S>(p + A.pos, v.x);
+        if (B.live) st_ring<S>(p + B.pos, v.y);
+      });
+    }
+    __syncthreads();
+    sp = (sp + 1) & 3;
+    sz = sz == 2 ? 0 : sz + 1;
+    sm = sm == R::kMinusSlots - 1 ? 0 : sm + 1;
+  }
+}
+
+// Second step of planes za .. zb - 1 (the block's other warps; t: thread
+// among them).
+template <int S, bool WALLS, bool FORCE, int CAP>
+__device__ __forceinline__ void step2_second(const typename Store<S>::T *__restrict__ ring,
+                                             const Dom2<S> &D, const PairConsts &C,
+                                             const float (&lidc)[Q], int x0, int y0, int cw,
+                                             int ch, int za, int zb, int t) {
+  using T = typename Store<S>::T;
+  using R = Ring<WALLS, CAP>;
+  const int lx_n = cw + 2;
+  const int n2 = cw * ch, half2 = cw * ((ch + 1) >> 1);
+  const int ia = t < n2 ? t : n2 - 1, ib = t + half2 < n2 ? t + half2 : n2 - 1;
+  const int ya = ia / cw, xa = ia - ya * cw, yb = ib / cw, xb = ib - yb * cw;
+  const int pa = (ya + 1) * lx_n + xa + 1, pb = (yb + 1) * lx_n + xb + 1;
+  const uint32_t oa = (uint32_t)(y0 + ya) * D.pitch + x0 + xa;
+  const uint32_t ob = (uint32_t)(y0 + yb) * D.pitch + x0 + xb;
+  const bool b_live = t + half2 < n2;
+  const uint32_t row = (uint32_t)D.ny * D.pitch;
+  const uint32_t drow = (uint32_t)D.ny * D.nx;
+  const bool wz = WALLS && (D.walls & LBM_WALL_Z);
+  uint32_t fa = 0, fb = 0;  // walled x and y faces of the two columns
+  if (WALLS && (D.walls & LBM_WALL_X)) {
+    fa |= (x0 + xa == 0 ? kX0 : 0u) | (x0 + xa == D.nx - 1 ? kX1 : 0u);
+    fb |= (x0 + xb == 0 ? kX0 : 0u) | (x0 + xb == D.nx - 1 ? kX1 : 0u);
+  }
+  if (WALLS && (D.walls & LBM_WALL_Y)) {
+    fa |= (y0 + ya == 0 ? kY0 : 0u) | (y0 + ya == D.ny - 1 ? kY1 : 0u);
+    fb |= (y0 + yb == 0 ? kY0 : 0u) | (y0 + yb == D.ny - 1 ? kY1 : 0u);
+  }
+  const uint32_t any = WALLS ? __reduce_or_sync(0xffffffffu, fa | fb) : 0u;
+
+  // plane za - 1 + j of the first step is in slots j modulo (4, 3, 2 or 3);
+  // the output plane za - 1 + j pulls from j - 1, j and j + 1
+  for (int k = 0; k < 3; ++k) __syncthreads();
+  int sp = 0, sz = 1, sm = WALLS ? 2 : 0;  // slots of j - 1, j, j + 1 at j = 1
+  for (int z = za; z < zb; ++z) {
+    if (t < half2) {
+      float da[Q], db[Q];
+      static_for<0, Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        constexpr int ex = kEx[i], ey = kEy[i];
+        const T *p = ring + R::template at<i>(sp, sz, sm);
+        da[i] = Store<S>::ld_smem(p + (pa - ey * lx_n - ex));
+        db[i] = Store<S>::ld_smem(p + (pb - ey * lx_n - ex));
+      });
+      const uint32_t zf = wz ? (z == 0 ? kZ0 : 0u) | (z == D.nz - 1 ? kZ1 : 0u) : 0u;
+      if (WALLS && (any | zf) != 0) {
+        // from beyond a wall: the opposite direction at the node itself, in
+        // its own plane's slots
+        const int sp1 = (sp + 1) & 3, sm1 = sm == 0 ? R::kMinusSlots - 1 : sm - 1;
+        for_bounces(fa | zf, any | zf, [&](auto I) {
+          constexpr int i = decltype(I)::value;
+          da[i] = Store<S>::ld_smem(ring + R::template at<kOpp_v<i>>(sp1, sz, sm1) + pa);
+        });
+        for_bounces(fb | zf, any | zf, [&](auto I) {
+          constexpr int i = decltype(I)::value;
+          db[i] = Store<S>::ld_smem(ring + R::template at<kOpp_v<i>>(sp1, sz, sm1) + pb);
+        });
+        if (zf & kZ1) {
+          static_for<1, Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            if constexpr (kEz[i] == -1) {
+              da[i] += lidc[i];
+              db[i] += lidc[i];
+            }
+          });
+        }
+      }
+      P2 d[Q];
+      static_for<0, Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        d[i] = pk(da[i], db[i]);
+      });
+      P2 rho, ux, uy, uz;
+      if constexpr (FORCE) {
+        const uint32_t ca = (uint32_t)z * drow + (uint32_t)(y0 + ya) * D.nx + (x0 + xa);
+        const uint32_t cb = (uint32_t)z * drow + (uint32_t)(y0 + yb) * D.nx + (x0 + xb);
+        collide_pair_force(d, D.omega, D.kf, D.force, D.cells, ca, cb, rho, ux, uy, uz);
+      } else {
+        collide_pair(d, C, rho, ux, uy, uz);
+      }
+      const uint32_t zoff = (uint32_t)z * row;
+      static_for<0, Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        const float2 v = unpk(d[i]);
+        Store<S>::st(D.fout[i] + (zoff + oa), v.x);
+        if (b_live) Store<S>::st(D.fout[i] + (zoff + ob), v.y);
+      });
+    }
+    if (z + 1 < zb) __syncthreads();
+    sp = (sp + 1) & 3;
+    sz = sz == 2 ? 0 : sz + 1;
+    sm = sm == R::kMinusSlots - 1 ? 0 : sm + 1;
+  }
+}
+
+}  // namespace lbm

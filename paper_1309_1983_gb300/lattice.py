@@ -133,6 +133,13 @@ class Lattice:
         launches; see lbm_set_graph_steps)."""
         capi.call("lbm_set_graph_steps", self._h, int(steps))
 
+    def set_fusion(self, mode):
+        """Two steps per launch in multi-step calls: "auto", "off" or
+        "always" (see lbm_set_fusion)."""
+        v = {"auto": capi.LBM_FUSE_AUTO, "off": capi.LBM_FUSE_OFF,
+             "always": capi.LBM_FUSE_ALWAYS}[mode]
+        capi.call("lbm_set_fusion", self._h, v)
+
     def set_wall_mode(self, mode):
         """"auto", "branch" or "select" (see lbm_set_wall_mode)."""
         v = {"auto": capi.LBM_WALLS_AUTO, "branch": capi.LBM_WALLS_BRANCH,

@@ -1,0 +1,97 @@
+"""Two steps per launch (lbm_set_fusion): the same bits as one step per
+launch of the two-node kernel, at the sizes where a tile, its rim, a chunk of
+planes or a remainder of steps can go wrong."""
+
+import numpy as np
+import pytest
+import torch
+
+from paper_1309_1983_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1309_1983_gb300 import build as B
+    B.build()
+
+
+GEOMS = {"periodic": ((0, 0, 0), None), "walls_x": ((1, 0, 0), None),
+         "walls_y": ((0, 1, 0), None), "walls_z": ((0, 0, 1), None),
+         "cavity": ((1, 1, 1), (0.05, 0.01, 0.0)), "lid_3d": ((0, 1, 1), (0.04, -0.02, 0.0))}
+# one node per axis, rows below and above a tile, several tiles with ragged
+# ends in x and y, many planes (several chunks) and two of them
+SHAPES = [(1, 7, 6), (5, 1, 1), (3, 2, 2), (37, 11, 9), (9, 61, 4), (129, 17, 5), (70, 45, 33),
+          (50, 33, 2), (8, 6, 400)]
+
+
+def _pair(shape, geom, storage, force):
+    """The state after 3 + 9 + 6 steps (groups of four and remainders), with
+    and without two steps per launch, and the buffer it ended in."""
+    from paper_1309_1983_gb300.lattice import Lattice
+    nx, ny, nz = shape
+    walls, lid = GEOMS[geom]
+    rho = torch.from_numpy(1 + W.noise((nz, ny, nx), 1, 0.03)).float().cuda()
+    u = torch.from_numpy(W.noise((3, nz, ny, nx), 2, 0.04)).float().cuda()
+    F = torch.from_numpy(W.noise((3, nz, ny, nx), 3, 1e-3)).float().cuda()
+    got = []
+    for mode in ("off", "always"):
+        L = Lattice(nx, ny, nz, 0.62, walls=tuple(bool(w) for w in walls), lid=lid,
+                    storage=storage, force=force)
+        L.set_fusion(mode)
+        if force:
+            L.force.copy_(F)
+        L.init_equilibrium(rho, u)
+        for n in (3, 9, 6):
+            L.step(n)
+        got.append((L.get_f(), L.current_buffers()[0].data_ptr() == L.f_a.data_ptr()))
+        L.close()
+    return got
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("geom", sorted(GEOMS))
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_same_bits_as_single_steps(shape, geom, storage):
+    for force in (False, True):
+        (ref, side), (f, fused_side) = _pair(shape, geom, storage, force)
+        np.testing.assert_array_equal(f, ref)
+        assert side == fused_side
+
+
+def test_default_takes_it_for_large_lattices():
+    """Above the line: the bits of single steps through graph replay,
+    plain launches and a last step that writes rho and u; and inside a stream
+    capture of the caller's."""
+    from paper_1309_1983_gb300.lattice import Lattice
+    dims = (83, 81, 67)  # 450,441 nodes
+    u = torch.from_numpy(W.noise((3,) + dims[::-1], 5, 0.04)).float().cuda()
+    outs = []
+    for mode in ("off", "auto"):
+        L = Lattice(*dims, 0.6, walls=(True, True, True), lid=(0.05, 0, 0))
+        L.set_fusion(mode)
+        L.init_equilibrium(u=u)
+        L.step(75)
+        rho, v = L.step_moments(7)
+        outs.append((L.get_f(), rho.cpu().numpy(), v.cpu().numpy()))
+        L.close()
+    for a, b in zip(*outs):
+        np.testing.assert_array_equal(a, b)
+
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        L = Lattice(*dims, 0.6, walls=(True, True, True), lid=(0.05, 0, 0), stream=s)
+        R = Lattice(*dims, 0.6, walls=(True, True, True), lid=(0.05, 0, 0), stream=s)
+        R.set_fusion("off")
+        for lat in (L, R):
+            lat.init_equilibrium(u=u)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            L.step(8)
+        for _ in range(3):
+            g.replay()
+        R.step(24)
+        torch.cuda.synchronize()
+    np.testing.assert_array_equal(L.get_f(), R.get_f())
