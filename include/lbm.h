@@ -484,6 +484,12 @@ int lbm_batch_set_timeout(lbm_batch_t *b, double seconds);
  * LBM_ETIMEOUT after the timeout instead of hanging. 0 restores normal use. */
 int lbm_batch_inject_barrier_fault(lbm_batch_t *b, int extra);
 
+/* Two steps per launch in lbm_batch_step, as lbm_set_fusion for a lattice
+ * (identical results; never while a barrier fault is injected). LBM_FUSE_AUTO
+ * (default): where both forms' modelled times say that it is faster, which is
+ * from about a million nodes on, and for a few small domains. */
+int lbm_batch_set_fusion(lbm_batch_t *b, int mode);
+
 /* Capture the persistent launch in a CUDA graph (default on) or launch it
  * directly (on = 0). */
 int lbm_batch_use_graph(lbm_batch_t *b, int on);
@@ -498,10 +504,12 @@ int lbm_batch_current(const lbm_batch_t *b, void **f_cur, void **f_other);
 /* Every domain to rest: f = w_i (rho = 1, u = 0). */
 int lbm_batch_init_rest(lbm_batch_t *b);
 
-/* n time steps of every domain in ONE persistent cooperative launch (a grid
- * barrier between steps, bounded waits), replayed from a CUDA graph. Waits
- * for the launch to finish; LBM_ETIMEOUT if a barrier wait ran out (the state
- * is then partly advanced and must be re-initialised). */
+/* n time steps of every domain: groups of four steps as ordinary launches of
+ * two steps each where lbm_batch_set_fusion allows it and they are faster,
+ * the others in ONE persistent cooperative launch (a grid barrier between
+ * steps, bounded waits), both replayed from CUDA graphs. Waits for the last
+ * launch to finish; LBM_ETIMEOUT if a barrier wait ran out (the state is then
+ * partly advanced and must be re-initialised). */
 int lbm_batch_step(lbm_batch_t *b, int n);
 
 /* The same n steps as n ordinary launches over the tile table (no grid

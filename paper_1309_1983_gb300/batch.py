@@ -88,6 +88,13 @@ class Batch:
     def inject_barrier_fault(self, extra):
         capi.call("lbm_batch_inject_barrier_fault", self._h, int(extra))
 
+    def set_fusion(self, mode):
+        """Two steps per launch in :meth:`step`: "auto", "off" or "always"
+        (see lbm_batch_set_fusion)."""
+        v = {"auto": capi.LBM_FUSE_AUTO, "off": capi.LBM_FUSE_OFF,
+             "always": capi.LBM_FUSE_ALWAYS}[mode]
+        capi.call("lbm_batch_set_fusion", self._h, v)
+
     def use_graph(self, on):
         capi.call("lbm_batch_use_graph", self._h, int(bool(on)))
 
@@ -133,7 +140,8 @@ class Batch:
         return res
 
     def step(self, n):
-        """n steps in one persistent launch (synchronises)."""
+        """n steps, two per launch or in one persistent launch
+        (synchronises)."""
         capi.call("lbm_batch_step", self._h, int(n))
 
     def step_launches(self, n):

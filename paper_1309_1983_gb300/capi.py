@@ -125,6 +125,7 @@ _SIGNATURES = {
     "lbm_batch_autotune": [_vp, ctypes.c_char_p, _i, _vp, _vp, _vp],
     "lbm_batch_set_timeout": [_vp, ctypes.c_double],
     "lbm_batch_inject_barrier_fault": [_vp, _i],
+    "lbm_batch_set_fusion": [_vp, _i],
     "lbm_batch_use_graph": [_vp, _i],
     "lbm_batch_info": [_vp, _vp, _vp, _vp, _vp],
     "lbm_batch_current": [_vp, ctypes.POINTER(_vp), ctypes.POINTER(_vp)],

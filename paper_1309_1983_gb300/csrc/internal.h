@@ -75,9 +75,15 @@ struct Step2Plan {
 // Whether multi-step calls of this lattice are faster so.
 bool step2_wins(int storage, int nx, int ny, int nz);
 // Once per handle and device before its launches.
-cudaError_t prepare_step2(int storage, const StepArgs &a);
+cudaError_t prepare_step2(int storage, const StepArgs &a, bool moments);
 Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms);
 cudaError_t launch_step2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s);
+// The same also writing the rho, u that both steps' collisions used (FP32).
+struct Moments2 {
+  float *rho[2], *u[2];
+};
+cudaError_t launch_step2_mom(const StepArgs &a, const Moments2 &m, const Step2Plan &p,
+                             cudaStream_t s);
 cudaError_t launch_step_pair16(int storage, bool moments, const StepArgs &a, int bxp, int by,
                                cudaStream_t s);
 // Four x-adjacent nodes per thread (bxq groups of four per block row, `by`
@@ -198,6 +204,16 @@ size_t batch_persistent_smem(int ndom);
 constexpr int kMaxBatchDomains = 256;  // table must fit in 48 KB of smem
 cudaError_t launch_batch_persistent(const BatchArgs &a, int grid, int threads,
                                     cudaStream_t s);
+// Two steps per launch (step2.cuh): a tile of a domain and a run [za, zb) of
+// its planes.
+struct Batch2Item {
+  int dom, x0, y0, cw, ch, za, zb, pad;
+};
+cudaError_t prepare_batch_step2(bool walls, bool moments);
+cudaError_t launch_batch_step2(const BatchArgs &a, const Batch2Item *items, int nitems,
+                               const float *fin, float *fout, const Moments2 &m, cudaStream_t s);
+// A tile size for an nx x ny domain, and the modelled time of one plane of it.
+void batch2_tile_of(int nx, int ny, int *w, int *h, double *plane_us);
 cudaError_t launch_batch_step(const BatchArgs &a, const float *fin, float *fout,
                               int threads, cudaStream_t s);
 // Persistent cooperative launches of a step sequence (grid barrier between

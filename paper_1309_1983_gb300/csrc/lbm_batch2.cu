@@ -1,0 +1,99 @@
+// lbm_batch2.cu - two steps of every domain of a batch per launch (step2.cuh).
+//
+// The persistent kernel moves 152 bytes per node and step and is within 6% of
+// the copy bandwidth (64 uneven cavities, 271 us a step); two steps per pass
+// halve the traffic, as for one lattice. One block per item: a tile of a
+// domain and a run of its planes. Items start longest first, so the uneven
+// domains finish together, and a domain's items follow one another, so that
+// neighbouring tiles find each other's rims in L2. A launch per pass in
+// place of a grid barrier: a pass takes 350 us there, a launch 2.
+//
+// The domains' relaxation rates differ, so the collision's constants come
+// from shared memory, and the planes are reached by 32-bit offsets from one
+// base: kernel parameters serve neither here.
+#include "internal.h"
+#include "step2.cuh"
+
+namespace lbm {
+
+using Slim = SlimBlock;
+
+template <bool WALLS, bool MOM>
+__global__ void __launch_bounds__(Slim::kThreads, 1)
+    k_batch_step2(const BatchArgs a, const Batch2Item *items, const float *fin, float *fout,
+                  const Moments2 m) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float *ring = reinterpret_cast<float *>(smem_raw);
+  __shared__ PairConsts consts;
+  const Batch2Item *ip = items + blockIdx.x;
+  if (!LBM_VALID(ip)) return;
+  const Batch2Item it = *ip;
+  if (!LBM_VALID(&a.doms[it.dom])) return;
+  const BatchDom &B = a.doms[it.dom];
+  BatchDom2 D;
+  D.fin = fin + B.foff;
+  D.fout = fout + B.foff;
+  D.force = nullptr;
+  for (int k = 0; k < 2; ++k) {
+    D.rho[k] = MOM ? m.rho[k] + B.coff : nullptr;
+    D.u[k] = MOM ? m.u[k] + 3 * (size_t)B.coff : nullptr;
+  }
+  D.nx = B.nx;
+  D.ny = B.ny;
+  D.nz = B.nz;
+  D.pitch = B.pitch;
+  D.plane = B.plane;
+  D.cells = B.cells;
+  D.walls = B.walls;
+  D.omega = B.omega;
+  D.kf = B.kf;
+  const int t = threadIdx.x;
+  if (t == 0) consts = pair_consts(B.omega);
+  __syncthreads();
+  if (t < Slim::kFirst) {
+    const bool side =
+        WALLS && (((D.walls & LBM_WALL_X) && (it.x0 <= 1 || it.x0 + it.cw >= D.nx - 1)) ||
+                  ((D.walls & LBM_WALL_Y) && (it.y0 <= 1 || it.y0 + it.ch >= D.ny - 1)));
+    if (side)
+      step2_first<0, WALLS ? 2 : 0, WALLS, false, MOM, Slim::kCap>(
+          ring, D, consts, B.lidc, it.x0, it.y0, it.cw, it.ch, it.za, it.zb, t);
+    else
+      step2_first<0, WALLS ? 1 : 0, WALLS, false, MOM, Slim::kCap>(
+          ring, D, consts, B.lidc, it.x0, it.y0, it.cw, it.ch, it.za, it.zb, t);
+  } else {
+    step2_second<0, WALLS, false, MOM, Slim::kCap>(ring, D, consts, B.lidc, it.x0, it.y0, it.cw,
+                                                  it.ch, it.za, it.zb, t - Slim::kFirst);
+  }
+}
+
+cudaError_t prepare_batch_step2(bool walls, bool moments) {
+  const void *k = walls ? (moments ? (const void *)k_batch_step2<true, true>
+                                   : (const void *)k_batch_step2<true, false>)
+                        : (moments ? (const void *)k_batch_step2<false, true>
+                                   : (const void *)k_batch_step2<false, false>);
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)step2_smem<Slim>(kF32, walls));
+}
+
+cudaError_t launch_batch_step2(const BatchArgs &a, const Batch2Item *items, int nitems,
+                               const float *fin, float *fout, const Moments2 &m, cudaStream_t s) {
+  const size_t smem = step2_smem<Slim>(kF32, a.walls_any != 0);
+  LBM_CHECK_TABLE(s, LBM_BATCH_RANGES(a), chk_r(items, (size_t)nitems * sizeof(Batch2Item)),
+                  chk_r(fin, LBM_BATCH_F(a)), chk_w(fout, LBM_BATCH_F(a)),
+                  chk_w(m.rho[0], LBM_BATCH_FIELD(a, 1)), chk_w(m.u[0], LBM_BATCH_FIELD(a, 3)),
+                  chk_w(m.rho[1], LBM_BATCH_FIELD(a, 1)), chk_w(m.u[1], LBM_BATCH_FIELD(a, 3)));
+  if (a.walls_any) {
+    if (m.rho[0])
+      k_batch_step2<true, true><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
+    else
+      k_batch_step2<true, false><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
+  } else {
+    if (m.rho[0])
+      k_batch_step2<false, true><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
+    else
+      k_batch_step2<false, false><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace lbm

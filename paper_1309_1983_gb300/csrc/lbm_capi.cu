@@ -188,7 +188,7 @@ bool fuses(const lbm_t *h) {
 // The two-step kernel's tiles, made before the first launch that needs them.
 int ensure_plan2(lbm_t *h) {
   if (h->plan2.w != 0 || !fuses(h)) return LBM_OK;
-  LBM_CUDA(lbm::prepare_step2(h->storage, make_args(h, nullptr, nullptr)), "two-step kernel setup");
+  LBM_CUDA(lbm::prepare_step2(h->storage, make_args(h, nullptr, nullptr), false), "two-step kernel setup");
   h->plan2 = lbm::step2_plan(h->storage, h->nx, h->ny, h->nz, h->sms);
   return LBM_OK;
 }

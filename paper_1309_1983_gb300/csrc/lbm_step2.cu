@@ -22,23 +22,18 @@
 // the next (60.3 against 65.3), and the 256-byte prefetch hint of the
 // single-step kernels (25.7: narrow tiles fetch their neighbours' values
 // several times over).
-#include "step2.cuh"
-
 #include <algorithm>
 
 #include "internal.h"
+#include "step2.cuh"
 
 namespace lbm {
 
-// Threads of the first step (two nodes each, so a tile with its rim has at
-// most kStep2Cap nodes) and of the second.
-constexpr int kFirst = 288, kSecond = 224;
-constexpr int kStep2Threads = kFirst + kSecond;
-constexpr int kStep2Cap = 2 * kFirst;
+using Wide = WideBlock;
 
 template <int S>
 struct Step2Args {
-  Dom2<S> dom;
+  PlanesDom<S> dom;
   PairConsts consts;
   float lidc[Q];
   Step2Plan plan;
@@ -47,11 +42,11 @@ struct Step2Args {
 // One block per tile and chunk of planes; blocks of one chunk are neighbours
 // in the grid, so that neighbouring tiles walk the same planes at the same
 // time and find each other's rims in L2.
-template <int S, bool WALLS, bool FORCE>
-__global__ void __launch_bounds__(kStep2Threads, 1)
+template <int S, bool WALLS, bool FORCE, bool MOM>
+__global__ void __launch_bounds__(Wide::kThreads, 1)
     k_step2(const __grid_constant__ Step2Args<S> a) {
   const Step2Plan &p = a.plan;
-  const Dom2<S> &D = a.dom;
+  const PlanesDom<S> &D = a.dom;
   using T = typename Store<S>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *ring = reinterpret_cast<T *>(smem_raw);
@@ -63,42 +58,67 @@ __global__ void __launch_bounds__(kStep2Threads, 1)
   const int zb = (int)((long long)D.nz * (chunk + 1) / p.chunks);
   const int cw = min(p.w, D.nx - x0), ch = min(p.h, D.ny - y0);
   const int t = threadIdx.x;
-  if (t < kFirst) {
+  if (t < Wide::kFirst) {
     // a tile away from the x and y walls takes the shorter form
     const bool side = WALLS && (((D.walls & LBM_WALL_X) && (x0 <= 1 || x0 + cw >= D.nx - 1)) ||
                                 ((D.walls & LBM_WALL_Y) && (y0 <= 1 || y0 + ch >= D.ny - 1)));
     if (side)
-      step2_first<S, WALLS ? 2 : 0, WALLS, FORCE, kStep2Cap>(ring, D, a.consts, a.lidc, x0, y0,
-                                                             cw, ch, za, zb, t);
+      step2_first<S, WALLS ? 2 : 0, WALLS, FORCE, MOM, Wide::kCap>(ring, D, a.consts, a.lidc, x0,
+                                                                  y0, cw, ch, za, zb, t);
     else
-      step2_first<S, WALLS ? 1 : 0, WALLS, FORCE, kStep2Cap>(ring, D, a.consts, a.lidc, x0, y0,
-                                                             cw, ch, za, zb, t);
+      step2_first<S, WALLS ? 1 : 0, WALLS, FORCE, MOM, Wide::kCap>(ring, D, a.consts, a.lidc, x0,
+                                                                  y0, cw, ch, za, zb, t);
   } else {
-    step2_second<S, WALLS, FORCE, kStep2Cap>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za, zb,
-                                             t - kFirst);
+    step2_second<S, WALLS, FORCE, MOM, Wide::kCap>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za,
+                                                  zb, t - Wide::kFirst);
   }
 }
 
-size_t step2_smem(int storage, bool walls) {
-  return (size_t)step2_ring_values(walls) * kStep2Cap * elem_bytes_of(storage);
+// Modelled time of one plane of a w x h tile: its traffic between L2 and the
+// SM. Per direction a row of the rim is read (with the sectors at its ends,
+// about 8 values more), a row of the tile written. Measured on tiles from
+// 8 x 54 to 64 x 12 with all SMs busy: 45 to 48 KB per us and SM.
+static double step2_plane_us(int bytes, int w, int h) {
+  const double kb = 0.019 * bytes * ((h + 2.0) * (w + 2 + 32 / bytes) + (double)h * w);
+  return std::max(0.1 + kb / 48.0, 0.9);
 }
 
-// The tile and the number of chunks with the least modelled time. One plane
-// of a tile takes the time of its traffic between L2 and the SM: per
-// direction a row of the rim is read (with the sectors at its ends, about 8
-// values more), a row of the tile written. Measured on tiles from 8 x 54 to
-// 64 x 12 with all SMs busy: 45 to 48 KB per us and SM. A chunk walks 3
-// planes more than it writes; the last wave of blocks counts in full.
+// Rows of the rim per thread that a tile of width w may have.
+template <class Block>
+static int step2_rows(int w) {
+  return std::min(Block::kFirst / (w + 2), Block::kSecond / w + 1);
+}
+
+// The tile of a batch domain whose columns cost least: equal shares of nx and
+// ny (the domains' rows are not padded, so no width is better aligned).
+void batch2_tile_of(int nx, int ny, int *w_out, int *h_out, double *plane_us) {
+  double best = 0.0;
+  for (int ntx = 1; ntx <= nx; ++ntx) {
+    const int w = (nx + ntx - 1) / ntx;
+    const int most = std::min(2 * step2_rows<SlimBlock>(w) - 2, ny);
+    if (w > SlimBlock::kSecond || most < 1) continue;
+    const int nty = (ny + most - 1) / most, h = (ny + nty - 1) / nty;
+    const double us = step2_plane_us(4, w, h);
+    if (best == 0.0 || us * ntx * nty < best) {
+      best = us * ntx * nty;
+      *w_out = w;
+      *h_out = h;
+      *plane_us = us;
+    }
+    if (w <= 8) break;
+  }
+}
+
+// The tile and the number of chunks with the least modelled time. A chunk
+// walks 3 planes more than it writes; the last wave of blocks counts in full.
 Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms) {
   Step2Plan best = {};
   const int bytes = elem_bytes_of(storage);
-  for (int w8 = 8; w8 < nx + 8 && w8 <= kSecond; w8 += 8) {
+  for (int w8 = 8; w8 < nx + 8 && w8 <= Wide::kSecond; w8 += 8) {
     const int w = w8 < nx ? w8 : nx;
-    const int rows = std::min(kFirst / (w + 2), kSecond / w + 1);  // of the rim, per thread
-    for (int h = std::min(2 * rows - 2, ny); h >= 1; --h) {
+    for (int h = std::min(2 * step2_rows<Wide>(w) - 2, ny); h >= 1; --h) {
       const int ntx = (nx + w - 1) / w, nty = (ny + h - 1) / h;
-      const double kb = 0.019 * bytes * ((h + 2.0) * (w + 2 + 32 / bytes) + (double)h * w);
-      const double plane_us = std::max(0.1 + kb / 48.0, 0.9);
+      const double plane_us = step2_plane_us(bytes, w, h);
       const long long tiles = (long long)ntx * nty;
       for (int k = 0; k <= 16; ++k) {  // chunks that fill k waves of blocks
         const int c = k == 0 ? 1 : (int)std::min<long long>(nz, (long long)k * sms / tiles);
@@ -113,16 +133,22 @@ Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms) {
   return best;
 }
 
-template <int S, bool WALLS, bool FORCE>
-static cudaError_t launch2(const StepArgs &a, const Step2Plan &p, size_t smem, cudaStream_t s) {
+template <int S, bool WALLS, bool FORCE, bool MOM>
+static cudaError_t launch2(const StepArgs &a, const Moments2 &m, const Step2Plan &p,
+                           cudaStream_t s) {
+  const size_t smem = step2_smem<Wide>(S, WALLS);
   if (p.w == 0)  // the plan's preparation: allow this much shared memory
-    return cudaFuncSetAttribute(k_step2<S, WALLS, FORCE>,
+    return cudaFuncSetAttribute(k_step2<S, WALLS, FORCE, MOM>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   Step2Args<S> b;
   for (int i = 0; i < Q; ++i) {
     b.dom.fin[i] = static_cast<const typename Store<S>::T *>(a.fin) + (size_t)i * a.plane;
     b.dom.fout[i] = static_cast<typename Store<S>::T *>(a.fout) + (size_t)i * a.plane;
     b.lidc[i] = a.lidc[i];
+  }
+  for (int k = 0; k < 2; ++k) {
+    b.dom.rho[k] = m.rho[k];
+    b.dom.u[k] = m.u[k];
   }
   b.dom.force = a.force;
   b.dom.nx = a.nx;
@@ -136,38 +162,51 @@ static cudaError_t launch2(const StepArgs &a, const Step2Plan &p, size_t smem, c
   b.dom.kf = a.kf;
   b.consts = pair_consts(a.omega);
   b.plan = p;
-  k_step2<S, WALLS, FORCE><<<p.ntx * p.nty * p.chunks, kStep2Threads, smem, s>>>(b);
+  k_step2<S, WALLS, FORCE, MOM>
+      <<<p.ntx * p.nty * p.chunks, Wide::kThreads, smem, s>>>(b);
   return cudaGetLastError();
 }
 
-static cudaError_t dispatch2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s) {
+static cudaError_t dispatch2(int storage, const StepArgs &a, const Moments2 &m, bool mom,
+                             const Step2Plan &p, cudaStream_t s) {
   const bool walls = a.walls != 0, force = a.force != nullptr;
-  const size_t smem = step2_smem(storage, walls);
-#define LBM_STEP2_CASE(S, W, F) \
-  if (storage == S && walls == W && force == F) return launch2<S, W, F>(a, p, smem, s);
-  LBM_STEP2_CASE(0, false, false)
-  LBM_STEP2_CASE(0, false, true)
-  LBM_STEP2_CASE(0, true, false)
-  LBM_STEP2_CASE(0, true, true)
-  LBM_STEP2_CASE(1, false, false)
-  LBM_STEP2_CASE(1, false, true)
-  LBM_STEP2_CASE(1, true, false)
-  LBM_STEP2_CASE(1, true, true)
-  LBM_STEP2_CASE(2, false, false)
-  LBM_STEP2_CASE(2, false, true)
-  LBM_STEP2_CASE(2, true, false)
-  LBM_STEP2_CASE(2, true, true)
+#define LBM_STEP2_CASE(S, W, F, M) \
+  if (storage == S && walls == W && force == F && mom == M) return launch2<S, W, F, M>(a, m, p, s);
+  LBM_STEP2_CASE(0, false, false, false)
+  LBM_STEP2_CASE(0, false, true, false)
+  LBM_STEP2_CASE(0, true, false, false)
+  LBM_STEP2_CASE(0, true, true, false)
+  LBM_STEP2_CASE(0, false, false, true)
+  LBM_STEP2_CASE(0, false, true, true)
+  LBM_STEP2_CASE(0, true, false, true)
+  LBM_STEP2_CASE(0, true, true, true)
+  LBM_STEP2_CASE(1, false, false, false)
+  LBM_STEP2_CASE(1, false, true, false)
+  LBM_STEP2_CASE(1, true, false, false)
+  LBM_STEP2_CASE(1, true, true, false)
+  LBM_STEP2_CASE(2, false, false, false)
+  LBM_STEP2_CASE(2, false, true, false)
+  LBM_STEP2_CASE(2, true, false, false)
+  LBM_STEP2_CASE(2, true, true, false)
 #undef LBM_STEP2_CASE
   return cudaErrorInvalidValue;
 }
 
-cudaError_t prepare_step2(int storage, const StepArgs &a) {
-  return dispatch2(storage, a, Step2Plan{}, nullptr);
+cudaError_t prepare_step2(int storage, const StepArgs &a, bool moments) {
+  return dispatch2(storage, a, Moments2{}, moments, Step2Plan{}, nullptr);
 }
 
 cudaError_t launch_step2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s) {
   LBM_CHECK_TABLE(s, LBM_STEP_RANGES(a, elem_bytes_of(storage)));
-  return dispatch2(storage, a, p, s);
+  return dispatch2(storage, a, Moments2{}, false, p, s);
+}
+
+cudaError_t launch_step2_mom(const StepArgs &a, const Moments2 &m, const Step2Plan &p,
+                             cudaStream_t s) {
+  LBM_CHECK_TABLE(s, LBM_STEP_RANGES(a, 4), chk_w(m.rho[0], (size_t)a.cells * 4),
+                  chk_w(m.u[0], 3 * (size_t)a.cells * 4), chk_w(m.rho[1], (size_t)a.cells * 4),
+                  chk_w(m.u[1], 3 * (size_t)a.cells * 4));
+  return dispatch2(kF32, a, m, true, p, s);
 }
 
 // Where two steps per launch are faster than two launches of the two-node

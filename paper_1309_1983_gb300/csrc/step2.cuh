@@ -25,6 +25,7 @@
 #pragma once
 
 #include "d3q19.cuh"
+#include "internal.h"
 #include "pair_math.cuh"
 #include "stream.cuh"
 
@@ -40,6 +41,23 @@ __host__ __device__ constexpr int ring_rank(int i) {
 // Values of shared memory per node of a tile with its rim.
 __host__ __device__ constexpr int step2_ring_values(bool walls) {
   return 4 * 5 + 3 * 9 + (walls ? 3 : 2) * 5;
+}
+
+// Threads of a block that take the first step (two nodes each, so a tile with
+// its rim has at most kCap nodes) and the second. Wide: 128 registers a
+// thread, for kernels whose constants are kernel parameters; Slim: 168.
+struct WideBlock {
+  static constexpr int kFirst = 288, kSecond = 224;
+  static constexpr int kThreads = kFirst + kSecond, kCap = 2 * kFirst;
+};
+struct SlimBlock {
+  static constexpr int kFirst = 224, kSecond = 160;
+  static constexpr int kThreads = kFirst + kSecond, kCap = 2 * kFirst;
+};
+
+template <class Block>
+size_t step2_smem(int storage, bool walls) {
+  return (size_t)step2_ring_values(walls) * Block::kCap * elem_bytes_of(storage);
 }
 
 // Store to shared memory in the storage type.
@@ -69,50 +87,127 @@ __device__ __forceinline__ P2 as_pair(const RawPair<S> &r) {
     return pk(__bfloat162float(r.a), __bfloat162float(r.b));
 }
 
-// One lattice of a two-step pass. The direction planes come as ready
-// pointers: in a kernel parameter they are constant-bank operands of the
-// address arithmetic, one instruction per access.
-template <int S>
-struct Dom2 {
-  using T = typename Store<S>::T;
-  const T *fin[Q];
-  T *fout[Q];
+// Geometry of a lattice in a two-step pass, and where its fields are. rho[k],
+// u[k]: density and velocity that step k's collision used (kernels with MOM).
+struct Geom2 {
   const float *force;  // dense [3][cells] or nullptr
+  float *rho[2], *u[2];
   int nx, ny, nz, pitch;
   uint32_t plane, cells, walls;
   float omega, kf;
 };
 
+// A lattice whose direction planes come as ready pointers: in a kernel
+// parameter they are constant-bank operands of the address arithmetic, one
+// instruction per access.
+template <int S>
+struct PlanesDom : Geom2 {
+  using T = typename Store<S>::T;
+  const T *fin[Q];
+  T *fout[Q];
+  __device__ __forceinline__ uint32_t stride() const { return 0; }
+  template <int i>
+  __device__ __forceinline__ const T *src(uint32_t off, uint32_t) const {
+    return fin[i] + off;
+  }
+  template <int i>
+  __device__ __forceinline__ T *dst(uint32_t off, uint32_t) const {
+    return fout[i] + off;
+  }
+};
+
+// A domain of a batch: the planes follow one another (at most 19 * 2^22
+// values, so 32-bit offsets from the first reach all of them).
+struct BatchDom2 : Geom2 {
+  const float *fin;
+  float *fout;
+  // The plane stride, taken anew for every plane of the walk: as a loop
+  // constant its 18 multiples would be kept in registers, and spilled.
+  __device__ __forceinline__ uint32_t stride() const {
+    uint32_t p = plane;
+    asm volatile("" : "+r"(p));
+    return p;
+  }
+  template <int i>
+  __device__ __forceinline__ const float *src(uint32_t off, uint32_t stride) const {
+    return fin + (i * stride + off);
+  }
+  template <int i>
+  __device__ __forceinline__ float *dst(uint32_t off, uint32_t stride) const {
+    return fout + (i * stride + off);
+  }
+};
+
+// rho and u of a node pair (a: node ca, b: node cb) into dense fields.
+__device__ __forceinline__ void store_moments(float *rho, float *u, uint32_t cells, uint32_t ca,
+                                              bool on_a, uint32_t cb, bool on_b, P2 r, P2 ux,
+                                              P2 uy, P2 uz) {
+  const float2 v[4] = {unpk(r), unpk(ux), unpk(uy), unpk(uz)};
+  float *u1 = u + cells, *u2 = u1 + cells;
+  if (on_a) {
+    LBM_ST(&rho[ca], v[0].x);
+    LBM_ST(&u[ca], v[1].x);
+    LBM_ST(&u1[ca], v[2].x);
+    LBM_ST(&u2[ca], v[3].x);
+  }
+  if (on_b) {
+    LBM_ST(&rho[cb], v[0].y);
+    LBM_ST(&u[cb], v[1].y);
+    LBM_ST(&u1[cb], v[2].y);
+    LBM_ST(&u2[cb], v[3].y);
+  }
+}
+
 // Walled faces a node touches.
 enum : uint32_t { kX0 = 1, kX1 = 2, kY0 = 4, kY1 = 8, kZ0 = 16, kZ1 = 32 };
 
-// In-plane part of a node of the first step: its place in the tile's ring
-// arrays and the wrapped neighbour offsets.
-struct Rim {
-  uint32_t yo[3], xo[3];  // (plus, same, minus) neighbour per axis
-  int pos;                // place in a ring plane
-  uint32_t fc;            // dense node of its force in an xy plane
-  uint32_t faces;         // walled x and y faces
-  bool live;              // the node exists (not beyond a wall)
+// Column of a node of the first step on the tile and its rim: the (plus, same,
+// minus) neighbours along x, wrapped.
+struct RimColumn {
+  uint32_t xo[3];
+  uint32_t faces;  // walled x faces
+  bool live;       // not beyond a wall
+  bool inner;      // a column of the tile
+};
+
+// Row of a node there: as above along y, and the node's place in a ring plane.
+struct RimRow {
+  uint32_t yo[3];
+  uint32_t faces;  // walled faces of the node
+  uint32_t fc;     // dense node in an xy plane
+  int pos;
+  bool live, inner;
 };
 
 template <bool WALLS>
-__device__ __forceinline__ Rim rim_node(int idx, int n, int lx_n, int x0, int y0, int cw, int ch,
-                                        int nx, int ny, int pitch, uint32_t walls) {
-  Rim r;
-  const int k = idx < n ? idx : n - 1;
-  const int ly = k / lx_n, lx = k - ly * lx_n;
-  r.pos = k;
-  r.live = idx < n;
-  int gx = x0 + lx - 1, gy = y0 + ly - 1;
+__device__ __forceinline__ RimColumn rim_column(int lx, int x0, int cw, int nx, uint32_t walls) {
+  RimColumn r;
+  int gx = x0 + lx - 1;
   r.faces = 0;
+  r.live = true;
   if (WALLS && (walls & LBM_WALL_X)) {
-    r.live &= gx >= 0 && gx < nx;
+    r.live = gx >= 0 && gx < nx;
     gx = min(max(gx, 0), nx - 1);
-    r.faces |= (gx == 0 ? kX0 : 0u) | (gx == nx - 1 ? kX1 : 0u);
+    r.faces = (gx == 0 ? kX0 : 0u) | (gx == nx - 1 ? kX1 : 0u);
   } else {
     gx = gx < 0 ? gx + nx : gx >= nx ? gx - nx : gx;
   }
+  r.inner = r.live && lx >= 1 && lx <= cw;
+  r.xo[0] = (uint32_t)(gx == nx - 1 ? 0 : gx + 1);
+  r.xo[1] = (uint32_t)gx;
+  r.xo[2] = (uint32_t)(gx == 0 ? nx - 1 : gx - 1);
+  return r;
+}
+
+template <bool WALLS>
+__device__ __forceinline__ RimRow rim_row(const RimColumn &c, int row, int lx, int lx_n, int y0,
+                                          int ch, int nx, int ny, int pitch, uint32_t walls) {
+  RimRow r;
+  const int ly = min(row, ch + 1);
+  int gy = y0 + ly - 1;
+  r.pos = ly * lx_n + lx;
+  r.faces = c.faces;
+  r.live = c.live && row < ch + 2;
   if (WALLS && (walls & LBM_WALL_Y)) {
     r.live &= gy >= 0 && gy < ny;
     gy = min(max(gy, 0), ny - 1);
@@ -120,16 +215,11 @@ __device__ __forceinline__ Rim rim_node(int idx, int n, int lx_n, int x0, int y0
   } else {
     gy = gy < 0 ? gy + ny : gy >= ny ? gy - ny : gy;
   }
-  if (!r.live) r.faces = 0;
-  r.fc = (uint32_t)gy * nx + gx;
-  const int xm = gx == 0 ? nx - 1 : gx - 1, xp = gx == nx - 1 ? 0 : gx + 1;
-  const int ym = gy == 0 ? ny - 1 : gy - 1, yp = gy == ny - 1 ? 0 : gy + 1;
-  r.xo[0] = (uint32_t)xp;
-  r.xo[1] = (uint32_t)gx;
-  r.xo[2] = (uint32_t)xm;
-  r.yo[0] = (uint32_t)yp * pitch;
+  r.inner = r.live && c.inner && ly >= 1 && ly <= ch;
+  r.fc = (uint32_t)gy * nx + c.xo[1];
+  r.yo[0] = (uint32_t)(gy == ny - 1 ? 0 : gy + 1) * pitch;
   r.yo[1] = (uint32_t)gy * pitch;
-  r.yo[2] = (uint32_t)ym * pitch;
+  r.yo[2] = (uint32_t)(gy == 0 ? ny - 1 : gy - 1) * pitch;
   return r;
 }
 
@@ -196,9 +286,9 @@ struct Ring {
 // First step of planes za - 1 .. zb on the tile and its rim (the block's
 // first warps; t: thread among them). FACES: the walls that the tile may
 // touch: 0 none, 1 z faces, 2 any.
-template <int S, int FACES, bool WALLS, bool FORCE, int CAP>
+template <int S, int FACES, bool WALLS, bool FORCE, bool MOM, int CAP, class Dom>
 __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ ring,
-                                            const Dom2<S> &D, const PairConsts &C,
+                                            const Dom &D, const PairConsts &C,
                                             const float (&lidc)[Q], int x0, int y0, int cw,
                                             int ch, int za, int zb, int t) {
   using T = typename Store<S>::T;
@@ -206,9 +296,11 @@ __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ r
   const int lx_n = cw + 2;
   // the two nodes of a thread lie in the same column, half the rows apart, so
   // that both touch an x wall or neither does
-  const int n1 = lx_n * (ch + 2), half1 = lx_n * ((ch + 3) >> 1);
-  const Rim A = rim_node<WALLS>(t, n1, lx_n, x0, y0, cw, ch, D.nx, D.ny, D.pitch, D.walls);
-  const Rim B = rim_node<WALLS>(t + half1, n1, lx_n, x0, y0, cw, ch, D.nx, D.ny, D.pitch, D.walls);
+  const int rows = (ch + 3) >> 1, half1 = lx_n * rows;
+  const int ly = min(t, half1 - 1) / lx_n, lx = min(t, half1 - 1) - ly * lx_n;
+  const RimColumn X = rim_column<WALLS>(lx, x0, cw, D.nx, D.walls);
+  const RimRow A = rim_row<WALLS>(X, ly, lx, lx_n, y0, ch, D.nx, D.ny, D.pitch, D.walls);
+  const RimRow B = rim_row<WALLS>(X, ly + rows, lx, lx_n, y0, ch, D.nx, D.ny, D.pitch, D.walls);
   const uint32_t row = (uint32_t)D.ny * D.pitch;
   const uint32_t drow = (uint32_t)D.ny * D.nx;
   const bool wz = WALLS && (D.walls & LBM_WALL_Z);
@@ -224,30 +316,30 @@ __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ r
     const uint32_t zo[3] = {(uint32_t)(z == D.nz - 1 ? 0 : z + 1) * row, (uint32_t)z * row,
                             (uint32_t)(z == 0 ? D.nz - 1 : z - 1) * row};
     const uint32_t zf = wz ? (z == 0 ? kZ0 : 0u) | (z == D.nz - 1 ? kZ1 : 0u) : 0u;
-    const uint32_t na = zo[1] + A.yo[1] + A.xo[1], nb = zo[1] + B.yo[1] + B.xo[1];
-    const uint32_t oa = na + D.plane, ob = nb + D.plane;
+    const uint32_t na = zo[1] + A.yo[1] + X.xo[1], nb = zo[1] + B.yo[1] + X.xo[1];
+    const uint32_t oa = na + D.plane, ob = nb + D.plane, ps = D.stride();
     static_for<0, Q>([&](auto I) {
       constexpr int i = decltype(I)::value;
       constexpr int jx = 1 + kEx[i], jy = 1 + kEy[i], jz = 1 + kEz[i];
       constexpr uint32_t mz = beyond_z(i), mxy = beyond_xy(i);
-      const uint32_t fa = zo[jz] + A.yo[jy] + A.xo[jx], fb = zo[jz] + B.yo[jy] + B.xo[jx];
+      const uint32_t fa = zo[jz] + A.yo[jy] + X.xo[jx], fb = zo[jz] + B.yo[jy] + X.xo[jx];
       if constexpr (FACES == 2 && (mz | mxy) != 0) {
         // opposite directions are neighbours (odd, even): both offsets count
         // from the odd one's plane, so a 32-bit selection picks the source
         constexpr bool even = i % 2 == 0;
-        const T *base = D.fin[even ? i - 1 : i];
+        constexpr int odd = even ? i - 1 : i;
         const bool ba = ((A.faces | zf) & (mz | mxy)) != 0;
         const bool bb = ((B.faces | zf) & (mz | mxy)) != 0;
-        d[i].a = LBM_LDGN(base + (even ? (ba ? na : fa + D.plane) : (ba ? oa : fa)));
-        d[i].b = LBM_LDGN(base + (even ? (bb ? nb : fb + D.plane) : (bb ? ob : fb)));
+        d[i].a = LBM_LDGN(D.template src<odd>(even ? (ba ? na : fa + D.plane) : (ba ? oa : fa), ps));
+        d[i].b = LBM_LDGN(D.template src<odd>(even ? (bb ? nb : fb + D.plane) : (bb ? ob : fb), ps));
       } else if constexpr (FACES == 1 && mz != 0) {
         const bool bz = (zf & mz) != 0;  // the same for all threads
-        const T *base = bz ? D.fin[kOpp_v<i>] : D.fin[i];
-        d[i].a = LBM_LDGN(base + (bz ? na : fa));
-        d[i].b = LBM_LDGN(base + (bz ? nb : fb));
+        constexpr int o = kOpp_v<i>;
+        d[i].a = LBM_LDGN(bz ? D.template src<o>(na, ps) : D.template src<i>(fa, ps));
+        d[i].b = LBM_LDGN(bz ? D.template src<o>(nb, ps) : D.template src<i>(fb, ps));
       } else {
-        d[i].a = LBM_LDGN(D.fin[i] + fa);
-        d[i].b = LBM_LDGN(D.fin[i] + fb);
+        d[i].a = LBM_LDGN(D.template src<i>(fa, ps));
+        d[i].b = LBM_LDGN(D.template src<i>(fb, ps));
       }
     });
   };
@@ -276,6 +368,12 @@ __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ r
       } else {
         collide_pair(d, C, rho, ux, uy, uz);
       }
+      if constexpr (MOM) {
+        const uint32_t zc = (uint32_t)z * drow;
+        const bool out = k >= 1 && k <= zb - za;  // not the planes of the rim
+        store_moments(D.rho[0], D.u[0], D.cells, zc + A.fc, out && A.inner, zc + B.fc,
+                      out && B.inner, rho, ux, uy, uz);
+      }
       static_for<0, Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         T *p = ring + R::template at<i>(sp, sz, sm);
@@ -293,28 +391,28 @@ __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ r
 
 // Second step of planes za .. zb - 1 (the block's other warps; t: thread
 // among them).
-template <int S, bool WALLS, bool FORCE, int CAP>
+template <int S, bool WALLS, bool FORCE, bool MOM, int CAP, class Dom>
 __device__ __forceinline__ void step2_second(const typename Store<S>::T *__restrict__ ring,
-                                             const Dom2<S> &D, const PairConsts &C,
+                                             const Dom &D, const PairConsts &C,
                                              const float (&lidc)[Q], int x0, int y0, int cw,
                                              int ch, int za, int zb, int t) {
   using T = typename Store<S>::T;
   using R = Ring<WALLS, CAP>;
   const int lx_n = cw + 2;
-  const int n2 = cw * ch, half2 = cw * ((ch + 1) >> 1);
-  const int ia = t < n2 ? t : n2 - 1, ib = t + half2 < n2 ? t + half2 : n2 - 1;
-  const int ya = ia / cw, xa = ia - ya * cw, yb = ib / cw, xb = ib - yb * cw;
-  const int pa = (ya + 1) * lx_n + xa + 1, pb = (yb + 1) * lx_n + xb + 1;
+  const int rows = (ch + 1) >> 1, half2 = cw * rows;
+  const int ya = min(t, half2 - 1) / cw, xa = min(t, half2 - 1) - ya * cw;
+  const bool b_live = ya + rows < ch;
+  const int yb = b_live ? ya + rows : ya;  // same column, half the rows up
+  const int pa = (ya + 1) * lx_n + xa + 1, pb = pa + (yb - ya) * lx_n;
   const uint32_t oa = (uint32_t)(y0 + ya) * D.pitch + x0 + xa;
-  const uint32_t ob = (uint32_t)(y0 + yb) * D.pitch + x0 + xb;
-  const bool b_live = t + half2 < n2;
+  const uint32_t ob = (uint32_t)(y0 + yb) * D.pitch + x0 + xa;
   const uint32_t row = (uint32_t)D.ny * D.pitch;
   const uint32_t drow = (uint32_t)D.ny * D.nx;
   const bool wz = WALLS && (D.walls & LBM_WALL_Z);
   uint32_t fa = 0, fb = 0;  // walled x and y faces of the two columns
   if (WALLS && (D.walls & LBM_WALL_X)) {
     fa |= (x0 + xa == 0 ? kX0 : 0u) | (x0 + xa == D.nx - 1 ? kX1 : 0u);
-    fb |= (x0 + xb == 0 ? kX0 : 0u) | (x0 + xb == D.nx - 1 ? kX1 : 0u);
+    fb |= (x0 + xa == 0 ? kX0 : 0u) | (x0 + xa == D.nx - 1 ? kX1 : 0u);
   }
   if (WALLS && (D.walls & LBM_WALL_Y)) {
     fa |= (y0 + ya == 0 ? kY0 : 0u) | (y0 + ya == D.ny - 1 ? kY1 : 0u);
@@ -367,17 +465,23 @@ __device__ __forceinline__ void step2_second(const typename Store<S>::T *__restr
       P2 rho, ux, uy, uz;
       if constexpr (FORCE) {
         const uint32_t ca = (uint32_t)z * drow + (uint32_t)(y0 + ya) * D.nx + (x0 + xa);
-        const uint32_t cb = (uint32_t)z * drow + (uint32_t)(y0 + yb) * D.nx + (x0 + xb);
+        const uint32_t cb = (uint32_t)z * drow + (uint32_t)(y0 + yb) * D.nx + (x0 + xa);
         collide_pair_force(d, D.omega, D.kf, D.force, D.cells, ca, cb, rho, ux, uy, uz);
       } else {
         collide_pair(d, C, rho, ux, uy, uz);
       }
-      const uint32_t zoff = (uint32_t)z * row;
+      if constexpr (MOM) {
+        const uint32_t zc = (uint32_t)z * drow;
+        store_moments(D.rho[1], D.u[1], D.cells, zc + (uint32_t)(y0 + ya) * D.nx + (x0 + xa),
+                      true, zc + (uint32_t)(y0 + yb) * D.nx + (x0 + xa), b_live, rho, ux, uy,
+                      uz);
+      }
+      const uint32_t zoff = (uint32_t)z * row, ps = D.stride();
       static_for<0, Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         const float2 v = unpk(d[i]);
-        Store<S>::st(D.fout[i] + (zoff + oa), v.x);
-        if (b_live) Store<S>::st(D.fout[i] + (zoff + ob), v.y);
+        Store<S>::st(D.template dst<i>(zoff + oa, ps), v.x);
+        if (b_live) Store<S>::st(D.template dst<i>(zoff + ob, ps), v.y);
       });
     }
     if (z + 1 < zb) __syncthreads();

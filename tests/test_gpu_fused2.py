@@ -95,3 +95,30 @@ def test_default_takes_it_for_large_lattices():
         R.step(24)
         torch.cuda.synchronize()
     np.testing.assert_array_equal(L.get_f(), R.get_f())
+
+
+BATCH_DIMS = [(17, 5, 9), (33, 16, 4), (1, 6, 7), (40, 3, 3), (8, 8, 8), (70, 45, 33), (5, 1, 1)]
+
+
+@pytest.mark.parametrize("walls", [(1, 1, 1), (0, 0, 0), (1, 0, 1), (0, 1, 0)])
+def test_batch_has_the_bits_of_single_steps(walls):
+    """Uneven domains, several tiles and runs of planes each; 39 steps are
+    graph replays, single passes and a remainder."""
+    from paper_1309_1983_gb300.batch import Batch
+    tau = [0.55, 0.7, 0.9, 1.0, 0.62, 0.6, 0.8]
+    lid = [0.02, 0.05, 0.08, 0.03, 0.06, 0.05, 0.04]
+    got = []
+    for mode in ("always", None):
+        B = Batch(BATCH_DIMS, tau, lid if walls[2] else None,
+                  walls=tuple(bool(w) for w in walls), lid=bool(walls[2]))
+        B.init_equilibrium(torch.from_numpy(W.noise(3 * B.cells, 7, 0.04)).float().cuda())
+        if mode:
+            B.set_fusion(mode)
+            B.step(39)
+        else:
+            B.step_launches(39)
+        got.append(([B.get_f(d) for d in range(len(BATCH_DIMS))],
+                    B.current_buffers()[0].data_ptr() == B.f_a.data_ptr()))
+    for d in range(len(BATCH_DIMS)):
+        np.testing.assert_array_equal(got[0][0][d], got[1][0][d])
+    assert got[0][1] == got[1][1]
