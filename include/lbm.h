@@ -303,6 +303,14 @@ int lbm_step_to(lbm_t *h, const void *f_in, void *f_out);
  * of lbm_adjoint_step_moments for this step. */
 int lbm_step_to_moments(lbm_t *h, const void *f_in, void *f_out, float *rho, float *u);
 
+/* n >= 1 steps from device buffer f_in into f_out (layout and storage as the
+ * bound ones), two steps per launch as lbm_set_fusion says. f_tmp, a third
+ * buffer, and f_out hold states in between; f_in is only read. rho and u:
+ * both NULL, or arrays of n device fields each that step k's collision writes
+ * (as lbm_step_to_moments). The bound pair is not touched. */
+int lbm_advance(lbm_t *h, int n, const void *f_in, void *f_out, void *f_tmp, float *const *rho,
+                float *const *u);
+
 /* Push iteration (Alg. 2) for the streaming-order comparison of Sec. 4.2:
  * g_in and g_out hold POST-STREAMING distributions (layout and storage as
  * the f buffers); each node reads its own values (aligned), collides, and
@@ -424,6 +432,13 @@ int lbm_adjoint_step(lbm_t *h, const void *f_n, const float *lambda_in,
  * rules and the same errors as lbm_adjoint_step. */
 int lbm_adjoint_step_moments(lbm_t *h, const float *rho_n, const float *u_n,
                              const float *lambda_in, float *lambda_out, float *grad_force);
+
+/* n >= 1 reverse steps from stored moments: step k reads lambda from lambda_a
+ * (k even) or lambda_b (k odd) and writes the other, with rho[k], u[k] the
+ * moments of the forward step it reverses (listed from the last forward step
+ * backwards). The result is in lambda_a if n is even, else in lambda_b. */
+int lbm_adjoint_run(lbm_t *h, int n, const float *const *rho, const float *const *u,
+                    float *lambda_a, float *lambda_b, float *grad_force);
 
 /* grad_u0 = sum_i lambda^0_i d f^eq_i(1, u0) / du0 (Eq. 5) for an initial
  * state f^0 = f^eq(1, u0); u0 may be NULL (zero velocity). Device buffers:
@@ -570,6 +585,11 @@ int lbm_batch_adjoint_u0(lbm_batch_t *b, const float *lambda0, const float *u0,
  * dense field the force cotangent is ADDED into. */
 int lbm_batch_run(lbm_batch_t *b, int n, const void *const *f_in, void *const *f_out,
                   float *const *rho, float *const *u);
+/* As lbm_advance, for every domain: two steps per launch where
+ * lbm_batch_set_fusion allows it and it is faster (asynchronous), else as
+ * lbm_batch_run in sequences of up to 64 steps (waits). */
+int lbm_batch_advance(lbm_batch_t *b, int n, const void *f_in, void *f_out, void *f_tmp,
+                      float *const *rho, float *const *u);
 int lbm_batch_adjoint_run(lbm_batch_t *b, int n, const float *const *rho, const float *const *u,
                           float *lambda_a, float *lambda_b, float *grad_force);
 

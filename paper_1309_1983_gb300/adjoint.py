@@ -8,8 +8,7 @@ lbm_adjoint_u0, or their lbm_batch_* counterparts for a batch of lattices).
 The forward keeps the states f^0, f^K, f^2K, ...; the backward recomputes
 each segment from its checkpoint and then runs the reverse steps over it.
 By default (``moments=True``) the recompute stores, per step, only the
-density and velocity its collision used (lbm_step_to_moments, 16 bytes per
-node): the collision Jacobian depends on the pulled state only through
+density and velocity its collision used (16 bytes per node): the collision Jacobian depends on the pulled state only through
 them, so the reverse step (lbm_adjoint_step_moments) reads those instead of
 re-gathering f^n, and a segment needs 16 instead of 76 bytes per node and
 step. ``moments=False`` keeps the K - 1 segment states and re-gathers them
@@ -63,12 +62,6 @@ class _Checkpointed:
     def _adj_step(self, fn, lam_in, lam_out, gF):
         raise NotImplementedError
 
-    def _step_mom(self, fin, fout, rho, u):
-        raise NotImplementedError
-
-    def _adj_step_mom(self, rho, u, lam_in, lam_out, gF):
-        raise NotImplementedError
-
     def _mom(self):  # (rho, u) buffers for one step
         raise NotImplementedError
 
@@ -81,22 +74,26 @@ class _Checkpointed:
     def _field(self):
         raise NotImplementedError
 
-    # -- step sequences: one call per step unless a subclass runs them in bulk --
-    def _run(self, fins, fouts):
-        for fin, fout in zip(fins, fouts):
-            self._step_to(fin, fout)
-
-    def _run_mom(self, fins, fouts, moms):
-        for fin, fout, (rho, u) in zip(fins, fouts, moms):
-            self._step_mom(fin, fout, rho, u)
+    # -- step sequences ----------------------------------------------------------
+    def _advance(self, fin, n, fout, tmp, moms=None):
+        """n steps from fin into fout (tmp: a third buffer), step k's
+        collision moments into moms[k]."""
+        raise NotImplementedError
 
     def _reverse(self, moms, lam_a, lam_b, gF):
         """Reverse steps over moms (last forward step first), lambda^{n+1} in
         lam_a; returns (lambda^n, the other buffer)."""
-        for rho, u in moms:
-            self._adj_step_mom(rho, u, lam_a, lam_b, gF)
-            lam_a, lam_b = lam_b, lam_a
-        return lam_a, lam_b
+        raise NotImplementedError
+
+    @staticmethod
+    def _ptrs(ts):
+        return (ctypes.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
+
+    def _moment_ptrs(self, moms):
+        """The rho and the u pointer arrays of a list of moment buffers."""
+        if moms is None:
+            return None, None
+        return self._ptrs([r for r, _ in moms]), self._ptrs([u for _, u in moms])
 
     # -- driver -------------------------------------------------------------------
     def _moment_buffers(self, m):
@@ -113,29 +110,23 @@ class _Checkpointed:
         if self._scratch is None:
             self._scratch = [self._fbuf(), self._fbuf()]
         self._tail_moments = False
-        f0 = self._init(u0, F)
-        ckpts = [f0]
-        prev = f0
-        fins, fouts = [], []
-        for n in range(1, self.T + 1):
-            if n % self.K == 0 and n < self.T:
+        prev = self._init(u0, F)
+        ckpts = [prev]
+        last, tmp = self._scratch
+        for start in range(0, self.T, self.K):  # one segment per call
+            m = min(self.K, self.T - start)
+            dst, moms = last, None
+            if start + m < self.T:
                 c = len(ckpts) - 1  # checkpoint buffers are reused across calls
                 if c == len(self._ckpt_pool):
                     self._ckpt_pool.append(self._fbuf())
                 dst = self._ckpt_pool[c]
                 ckpts.append(dst)
-            else:
-                dst = self._scratch[n % 2]
-            fins.append(prev)
-            fouts.append(dst)
+            elif keep_tail and self.moments:
+                moms = self._moment_buffers(m)
+                self._tail_moments = True
+            self._advance(prev, m, dst, tmp, moms)
             prev = dst
-            if n % self.K == 0 or n == self.T:  # one segment per call
-                if n == self.T and keep_tail and self.moments:
-                    self._run_mom(fins, fouts, self._moment_buffers(len(fins)))
-                    self._tail_moments = True
-                else:
-                    self._run(fins, fouts)
-                fins, fouts = [], []
         return prev, ckpts
 
     def backward(self, f_T, ckpts, u0, ut):
@@ -157,9 +148,7 @@ class _Checkpointed:
                 # f_T (a scratch buffer) is no longer needed after the seed
                 m = stop - start
                 if not (self._tail_moments and s == len(ckpts) - 1):
-                    fins = [ckpts[s]] + [self._scratch[k % 2] for k in range(m - 1)]
-                    fouts = [self._scratch[k % 2] for k in range(m)]
-                    self._run_mom(fins, fouts, self._mom_seg[:m])
+                    self._advance(ckpts[s], m, *self._scratch, self._mom_seg[:m])
                 lam_a, lam_b = self._reverse(self._mom_seg[:m][::-1], lam_a, lam_b, gF)
                 continue
             states = [ckpts[s]]
@@ -228,12 +217,15 @@ class AdjointProblem(_Checkpointed):
     def _adj_step(self, fn, lam_in, lam_out, gF):
         capi.call("lbm_adjoint_step", self.lat.handle, _p(fn), _p(lam_in), _p(lam_out), _p(gF))
 
-    def _step_mom(self, fin, fout, rho, u):
-        capi.call("lbm_step_to_moments", self.lat.handle, _p(fin), _p(fout), _p(rho), _p(u))
+    def _advance(self, fin, n, fout, tmp, moms=None):
+        rho, u = self._moment_ptrs(moms)
+        capi.call("lbm_advance", self.lat.handle, n, _p(fin), _p(fout), _p(tmp), rho, u)
 
-    def _adj_step_mom(self, rho, u, lam_in, lam_out, gF):
-        capi.call("lbm_adjoint_step_moments", self.lat.handle, _p(rho), _p(u), _p(lam_in),
-                  _p(lam_out), _p(gF))
+    def _reverse(self, moms, lam_a, lam_b, gF):
+        rho, u = self._moment_ptrs(moms)
+        capi.call("lbm_adjoint_run", self.lat.handle, len(moms), rho, u, _p(lam_a), _p(lam_b),
+                  _p(gF))
+        return (lam_b, lam_a) if len(moms) % 2 else (lam_a, lam_b)
 
     def _mom(self):
         return (torch.empty(self.shape, dtype=torch.float32, device=self.device),
@@ -279,13 +271,6 @@ class BatchAdjointProblem(_Checkpointed):
         capi.call("lbm_batch_adjoint_step", self.b.handle, _p(fn), _p(lam_in), _p(lam_out),
                   _p(gF))
 
-    def _step_mom(self, fin, fout, rho, u):
-        capi.call("lbm_batch_step_to_moments", self.b.handle, _p(fin), _p(fout), _p(rho), _p(u))
-
-    def _adj_step_mom(self, rho, u, lam_in, lam_out, gF):
-        capi.call("lbm_batch_adjoint_step_moments", self.b.handle, _p(rho), _p(u), _p(lam_in),
-                  _p(lam_out), _p(gF))
-
     def _mom(self):
         return (torch.empty(self.b.cells, dtype=torch.float32, device=self.device),
                 torch.empty(3 * self.b.cells, dtype=torch.float32, device=self.device))
@@ -299,32 +284,19 @@ class BatchAdjointProblem(_Checkpointed):
     def _field(self):
         return torch.empty(3 * self.b.cells, dtype=torch.float32, device=self.device)
 
-    # segments, recompute and reverse sweeps as persistent launches of up to
-    # 64 steps each (lbm_batch_run, lbm_batch_adjoint_run)
+    def _advance(self, fin, n, fout, tmp, moms=None):
+        rho, u = self._moment_ptrs(moms)
+        capi.call("lbm_batch_advance", self.b.handle, n, _p(fin), _p(fout), _p(tmp), rho, u)
+
+    # reverse sweeps as persistent launches of up to 64 steps each
     _CHUNK = 64
-
-    @staticmethod
-    def _ptrs(ts):
-        return (ctypes.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
-
-    def _run(self, fins, fouts):
-        for k in range(0, len(fins), self._CHUNK):
-            fi, fo = fins[k:k + self._CHUNK], fouts[k:k + self._CHUNK]
-            capi.call("lbm_batch_run", self.b.handle, len(fi), self._ptrs(fi), self._ptrs(fo),
-                      None, None)
-
-    def _run_mom(self, fins, fouts, moms):
-        for k in range(0, len(fins), self._CHUNK):
-            fi, fo, mm = fins[k:k + self._CHUNK], fouts[k:k + self._CHUNK], moms[k:k + self._CHUNK]
-            capi.call("lbm_batch_run", self.b.handle, len(fi), self._ptrs(fi), self._ptrs(fo),
-                      self._ptrs([r for r, _ in mm]), self._ptrs([u for _, u in mm]))
 
     def _reverse(self, moms, lam_a, lam_b, gF):
         for k in range(0, len(moms), self._CHUNK):
             mm = moms[k:k + self._CHUNK]
-            capi.call("lbm_batch_adjoint_run", self.b.handle, len(mm),
-                      self._ptrs([r for r, _ in mm]), self._ptrs([u for _, u in mm]),
-                      _p(lam_a), _p(lam_b), _p(gF))
+            rho, u = self._moment_ptrs(mm)
+            capi.call("lbm_batch_adjoint_run", self.b.handle, len(mm), rho, u, _p(lam_a),
+                      _p(lam_b), _p(gF))
             if len(mm) % 2:
                 lam_a, lam_b = lam_b, lam_a
         return lam_a, lam_b

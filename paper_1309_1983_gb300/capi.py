@@ -104,6 +104,7 @@ _SIGNATURES = {
     "lbm_step_moments": [_vp, _i, _vp, _vp],
     "lbm_step_to": [_vp, _vp, _vp],
     "lbm_step_to_moments": [_vp, _vp, _vp, _vp, _vp],
+    "lbm_advance": [_vp, _i, _vp, _vp, _vp, _vp, _vp],
     "lbm_step_push": [_vp, _vp, _vp],
     "lbm_stream": [_vp, _vp, _vp, _i],
     "lbm_moments": [_vp, _vp, _vp, _dp],
@@ -116,6 +117,7 @@ _SIGNATURES = {
     "lbm_adjoint_seed": [_vp, _vp, _vp, _vp, _vp, _vp],
     "lbm_adjoint_step": [_vp, _vp, _vp, _vp, _vp],
     "lbm_adjoint_step_moments": [_vp, _vp, _vp, _vp, _vp, _vp],
+    "lbm_adjoint_run": [_vp, _i, _vp, _vp, _vp, _vp, _vp],
     "lbm_adjoint_u0": [_vp, _vp, _vp, _vp],
     "lbm_batch_create": [_i, _vp, _vp, _vp, _u32, ctypes.POINTER(_vp)],
     "lbm_batch_destroy": [_vp],
@@ -143,6 +145,7 @@ _SIGNATURES = {
     "lbm_batch_adjoint_step_moments": [_vp, _vp, _vp, _vp, _vp, _vp],
     "lbm_batch_adjoint_u0": [_vp, _vp, _vp, _vp],
     "lbm_batch_run": [_vp, _i, _vp, _vp, _vp, _vp],
+    "lbm_batch_advance": [_vp, _i, _vp, _vp, _vp, _vp, _vp],
     "lbm_batch_adjoint_run": [_vp, _i, _vp, _vp, _vp, _vp, _vp],
     "lbm_check_status": [_vp, _vp, _vp, _vp],
     "lbm_check_reset": [],

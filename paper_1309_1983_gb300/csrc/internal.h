@@ -76,7 +76,7 @@ struct Step2Plan {
 bool step2_wins(int storage, int nx, int ny, int nz);
 // Once per handle and device before its launches.
 cudaError_t prepare_step2(int storage, const StepArgs &a, bool moments);
-Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms);
+Step2Plan step2_plan(int storage, bool force, bool moments, int nx, int ny, int nz, int sms);
 cudaError_t launch_step2(int storage, const StepArgs &a, const Step2Plan &p, cudaStream_t s);
 // The same also writing the rho, u that both steps' collisions used (FP32).
 struct Moments2 {
@@ -263,7 +263,8 @@ struct lbm_lattice {
   int fuse;      // LBM_FUSE_AUTO / OFF / ALWAYS
   int wall_mode; // LBM_WALLS_AUTO / BRANCH / SELECT
   int sms;       // SM count of the bound device
-  lbm::Step2Plan plan2;  // tiles of the two-step kernel (w = 0: not made yet)
+  // tiles of the two-step kernel, without and with moments (w = 0: not made yet)
+  lbm::Step2Plan plan2[2];
   int pbx, pby;  // block shape of the pair kernel (pairs along x, rows)
   int device;
   lbm::Scratch scr;

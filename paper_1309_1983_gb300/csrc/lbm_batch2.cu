@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(Slim::kThreads, 1)
   D.omega = B.omega;
   D.kf = B.kf;
   const int t = threadIdx.x;
-  if (t == 0) consts = pair_consts(B.omega);
+  if (t == 0) consts = pair_consts(B.omega, B.kf);
   __syncthreads();
   if (t < Slim::kFirst) {
     const bool side =

@@ -818,6 +818,60 @@ int lbm_batch_run(lbm_batch_t *b, int n, const void *const *f_in, void *const *f
   });
 }
 
+int lbm_batch_advance(lbm_batch_t *b, int n, const void *f_in, void *f_out, void *f_tmp,
+                      float *const *rho, float *const *u) {
+  LBM_BREQUIRE_ALIGNED(aligned_to(f_in, kAlignF) && aligned_to(f_out, kAlignF) &&
+                       aligned_to(f_tmp, kAlignF));
+  for (int k = 0; rho && u && k < n; ++k)
+    LBM_BREQUIRE_ALIGNED(aligned_to(rho[k], kAlignField) && aligned_to(u[k], kAlignField));
+  int rc = check_b(b);
+  if (rc) return rc;
+  if (n < 1 || !f_in || !f_out || !f_tmp || f_in == f_out || f_in == f_tmp || f_out == f_tmp)
+    return bfail(LBM_EINVAL, "need n >= 1 and three distinct f buffers");
+  if ((rho == nullptr) != (u == nullptr)) return bfail(LBM_EINVAL, "give both rho and u or neither");
+  for (int k = 0; rho && k < n; ++k)
+    if (!rho[k] || !u[k]) return bfail(LBM_EINVAL, "NULL rho or u buffer");
+  bool pair = n >= 2 && b->inject_extra == 0 && b->fuse != LBM_FUSE_OFF;
+  if (pair && (rc = upload_items(b))) return rc;
+  pair = pair && pairs_win(b);
+  // passes of two steps and a last one of one, or of one step each; they
+  // alternate between the two buffers and end in f_out
+  const int per = pair ? 2 : 1;
+  const int passes = (n + per - 1) / per;
+  std::vector<const void *> in(passes);
+  std::vector<void *> out(passes);
+  for (int p = 0; p < passes; ++p) {
+    out[p] = (passes - p) % 2 ? f_out : f_tmp;
+    in[p] = p == 0 ? f_in : out[p - 1];
+  }
+  if (!pair) {
+    for (int k = 0; k < n; k += lbm::kMaxSeqSteps) {
+      const int m = std::min(lbm::kMaxSeqSteps, n - k);
+      rc = lbm_batch_run(b, m, &in[k], &out[k], rho ? rho + k : nullptr, u ? u + k : nullptr);
+      if (rc) return rc;
+    }
+    return LBM_OK;
+  }
+  const BatchArgs a = make_args(b);
+  for (int p = 0; p < passes; ++p) {
+    const float *fi = static_cast<const float *>(in[p]);
+    float *fo = static_cast<float *>(out[p]);
+    const int k = 2 * p;
+    cudaError_t e;
+    if (k + 1 < n) {
+      lbm::Moments2 m = {};
+      if (rho) m = {{rho[k], rho[k + 1]}, {u[k], u[k + 1]}};
+      e = lbm::launch_batch_step2(a, b->d_items, b->nitems, fi, fo, m, b->stream);
+    } else if (rho) {
+      e = lbm::launch_batch_step_mom(a, fi, fo, rho[k], u[k], b->threads, b->stream);
+    } else {
+      e = lbm::launch_batch_step(a, fi, fo, b->threads, b->stream);
+    }
+    BCUDA(e, "batch advance launch");
+  }
+  return LBM_OK;
+}
+
 int lbm_batch_adjoint_run(lbm_batch_t *b, int n, const float *const *rho, const float *const *u,
                           float *lambda_a, float *lambda_b, float *grad_force) {
   int rc = check_b(b);

@@ -186,10 +186,13 @@ bool fuses(const lbm_t *h) {
 }
 
 // The two-step kernel's tiles, made before the first launch that needs them.
-int ensure_plan2(lbm_t *h) {
-  if (h->plan2.w != 0 || !fuses(h)) return LBM_OK;
-  LBM_CUDA(lbm::prepare_step2(h->storage, make_args(h, nullptr, nullptr), false), "two-step kernel setup");
-  h->plan2 = lbm::step2_plan(h->storage, h->nx, h->ny, h->nz, h->sms);
+int ensure_plan2(lbm_t *h, bool moments) {
+  lbm::Step2Plan &p = h->plan2[moments];
+  if (p.w != 0 || !fuses(h)) return LBM_OK;
+  LBM_CUDA(lbm::prepare_step2(h->storage, make_args(h, nullptr, nullptr), moments),
+           "two-step kernel setup");
+  p = lbm::step2_plan(h->storage, (h->flags & LBM_FORCE) != 0, moments, h->nx, h->ny, h->nz,
+                      h->sms);
   return LBM_OK;
 }
 
@@ -202,7 +205,7 @@ cudaError_t enqueue_steps(const lbm_t *h, int n, int c, cudaStream_t s, int *c_e
   if (fuses(h))
     for (; n >= 4 && e == cudaSuccess; n -= 4)
       for (int k = 0; k < 2 && e == cudaSuccess; ++k, c ^= 1)
-        e = lbm::launch_step2(h->storage, make_args(h, h->f[c], h->f[1 - c]), h->plan2, s);
+        e = lbm::launch_step2(h->storage, make_args(h, h->f[c], h->f[1 - c]), h->plan2[0], s);
   for (; n > 0 && e == cudaSuccess; --n, c ^= 1)
     e = launch_one_step(h, false, make_args(h, h->f[c], h->f[1 - c]), s);
   *c_end = c;
@@ -284,7 +287,7 @@ void release_pipeline(lbm_t *h) {
 }
 
 int do_steps(lbm_t *h, int n, float *rho, float *u) {
-  int rc = ensure_plan2(h);
+  int rc = ensure_plan2(h, false);
   if (rc) return rc;
   // whole graphs first (an even number of steps each, so the current buffer
   // is unchanged), then plain launches; a step writing rho, u is always plain
@@ -500,7 +503,7 @@ int lbm_bind(lbm_t *h, void *f_a, void *f_b, const float *force, void *stream) {
   if (force && !aligned(force, 4)) return fail(LBM_EINVAL, "force misaligned");
   int rc = ensure_scratch(h);
   if (rc) return rc;
-  h->plan2 = lbm::Step2Plan{};
+  h->plan2[0] = h->plan2[1] = lbm::Step2Plan{};
   h->f[0] = f_a;
   h->f[1] = f_b;
   h->cur = 0;
@@ -650,6 +653,48 @@ int lbm_step_to_moments(lbm_t *h, const void *f_in, void *f_out, float *rho, flo
   a.u = u;
   cudaError_t e = launch_one_step(h, true, a);
   if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+  return LBM_OK;
+}
+
+int lbm_advance(lbm_t *h, int n, const void *f_in, void *f_out, void *f_tmp, float *const *rho,
+                float *const *u) {
+  LBM_REQUIRE_ALIGNED(aligned(f_in, kAlignF) && aligned(f_out, kAlignF) && aligned(f_tmp, kAlignF));
+  for (int k = 0; rho && u && k < n; ++k)
+    LBM_REQUIRE_ALIGNED(aligned(rho[k], kAlignField) && aligned(u[k], kAlignField));
+  int rc = check_bound(h);
+  if (rc) return rc;
+  if (n < 1 || !f_in || !f_out || !f_tmp || f_in == f_out || f_in == f_tmp || f_out == f_tmp)
+    return fail(LBM_EINVAL, "need n >= 1 and three distinct f buffers");
+  if ((rho == nullptr) != (u == nullptr)) return fail(LBM_EINVAL, "give both rho and u or neither");
+  for (int k = 0; rho && k < n; ++k)
+    if (!rho[k] || !u[k]) return fail(LBM_EINVAL, "NULL rho or u buffer");
+  if (!rho || h->storage == lbm::kF32) rc = ensure_plan2(h, rho != nullptr);
+  if (rc) return rc;
+  const int pairs = fuses(h) && (!rho || h->storage == lbm::kF32) ? n / 2 : 0;
+  int left = pairs + (n - 2 * pairs);  // passes; they alternate and end in f_out
+  const void *in = f_in;
+  for (int k = 0; k < n; --left) {
+    void *out = left % 2 ? f_out : f_tmp;
+    StepArgs a = make_args(h, in, out);
+    cudaError_t e;
+    if (k < 2 * pairs) {
+      if (rho)
+        e = lbm::launch_step2_mom(a, {{rho[k], rho[k + 1]}, {u[k], u[k + 1]}}, h->plan2[1],
+                                  h->stream);
+      else
+        e = lbm::launch_step2(h->storage, a, h->plan2[0], h->stream);
+      k += 2;
+    } else {
+      if (rho) {
+        a.rho = rho[k];
+        a.u = u[k];
+      }
+      e = launch_one_step(h, rho != nullptr, a);
+      ++k;
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
+    in = out;
+  }
   return LBM_OK;
 }
 
@@ -953,6 +998,18 @@ int lbm_adjoint_step_moments(lbm_t *h, const float *rho_n, const float *u_n,
   cudaError_t e = lbm::launch_adjoint_step_mom(g, rho_n, u_n, lambda_in, lambda_out, grad_force,
                                                abx, 128 / abx, h->stream);
   if (e != cudaSuccess) return cuda_fail(e, "adjoint step launch");
+  return LBM_OK;
+}
+
+int lbm_adjoint_run(lbm_t *h, int n, const float *const *rho, const float *const *u,
+                    float *lambda_a, float *lambda_b, float *grad_force) {
+  if (!h) return fail(LBM_EINVAL, "NULL handle");
+  if (n < 1 || !rho || !u) return fail(LBM_EINVAL, "need n >= 1 and the rho, u arrays");
+  for (int k = 0; k < n; ++k) {
+    const int rc = lbm_adjoint_step_moments(h, rho[k], u[k], k % 2 ? lambda_b : lambda_a,
+                                            k % 2 ? lambda_a : lambda_b, grad_force);
+    if (rc) return rc;
+  }
   return LBM_OK;
 }
 

@@ -14,7 +14,9 @@
 // 16-bit storage moves half the bytes, so there the two collisions and the
 // conversions bound the pass.
 //
-// One block per SM of 9 + 7 warps at 128 registers. Tried and slower, 384^3
+// One block per SM of 9 + 7 warps at 128 registers (7 + 5 at 168 with a body
+// force or moments, which spill at 128: 256^3 periodic with both 435 / 340 us
+// a step). Tried and slower, 384^3
 // periodic FP32: all warps alternating between the two steps with a barrier
 // after each (48.6 without, 65.3 with the next plane's loads in flight over
 // the second step), 11 + 9 warps at 96 registers (59.9, spills), 7 + 5 at
@@ -23,13 +25,18 @@
 // single-step kernels (25.7: narrow tiles fetch their neighbours' values
 // several times over).
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "step2.cuh"
 
 namespace lbm {
 
-using Wide = WideBlock;
+// Body force and moments need more registers than the wide block has (128^3
+// with both 90.6 us a step there, 52.8 in the slim one; without either 35.7
+// and 42.6).
+template <bool FORCE, bool MOM>
+using BlockOf = std::conditional_t<FORCE || MOM, SlimBlock, WideBlock>;
 
 template <int S>
 struct Step2Args {
@@ -43,8 +50,9 @@ struct Step2Args {
 // in the grid, so that neighbouring tiles walk the same planes at the same
 // time and find each other's rims in L2.
 template <int S, bool WALLS, bool FORCE, bool MOM>
-__global__ void __launch_bounds__(Wide::kThreads, 1)
+__global__ void __launch_bounds__(BlockOf<FORCE, MOM>::kThreads, 1)
     k_step2(const __grid_constant__ Step2Args<S> a) {
+  using Block = BlockOf<FORCE, MOM>;
   const Step2Plan &p = a.plan;
   const PlanesDom<S> &D = a.dom;
   using T = typename Store<S>::T;
@@ -58,19 +66,19 @@ __global__ void __launch_bounds__(Wide::kThreads, 1)
   const int zb = (int)((long long)D.nz * (chunk + 1) / p.chunks);
   const int cw = min(p.w, D.nx - x0), ch = min(p.h, D.ny - y0);
   const int t = threadIdx.x;
-  if (t < Wide::kFirst) {
+  if (t < Block::kFirst) {
     // a tile away from the x and y walls takes the shorter form
     const bool side = WALLS && (((D.walls & LBM_WALL_X) && (x0 <= 1 || x0 + cw >= D.nx - 1)) ||
                                 ((D.walls & LBM_WALL_Y) && (y0 <= 1 || y0 + ch >= D.ny - 1)));
     if (side)
-      step2_first<S, WALLS ? 2 : 0, WALLS, FORCE, MOM, Wide::kCap>(ring, D, a.consts, a.lidc, x0,
+      step2_first<S, WALLS ? 2 : 0, WALLS, FORCE, MOM, Block::kCap>(ring, D, a.consts, a.lidc, x0,
                                                                   y0, cw, ch, za, zb, t);
     else
-      step2_first<S, WALLS ? 1 : 0, WALLS, FORCE, MOM, Wide::kCap>(ring, D, a.consts, a.lidc, x0,
+      step2_first<S, WALLS ? 1 : 0, WALLS, FORCE, MOM, Block::kCap>(ring, D, a.consts, a.lidc, x0,
                                                                   y0, cw, ch, za, zb, t);
   } else {
-    step2_second<S, WALLS, FORCE, MOM, Wide::kCap>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za,
-                                                  zb, t - Wide::kFirst);
+    step2_second<S, WALLS, FORCE, MOM, Block::kCap>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za,
+                                                  zb, t - Block::kFirst);
   }
 }
 
@@ -111,12 +119,13 @@ void batch2_tile_of(int nx, int ny, int *w_out, int *h_out, double *plane_us) {
 
 // The tile and the number of chunks with the least modelled time. A chunk
 // walks 3 planes more than it writes; the last wave of blocks counts in full.
-Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms) {
+template <class Block>
+static Step2Plan plan_for(int storage, int nx, int ny, int nz, int sms) {
   Step2Plan best = {};
   const int bytes = elem_bytes_of(storage);
-  for (int w8 = 8; w8 < nx + 8 && w8 <= Wide::kSecond; w8 += 8) {
+  for (int w8 = 8; w8 < nx + 8 && w8 <= Block::kSecond; w8 += 8) {
     const int w = w8 < nx ? w8 : nx;
-    for (int h = std::min(2 * step2_rows<Wide>(w) - 2, ny); h >= 1; --h) {
+    for (int h = std::min(2 * step2_rows<Block>(w) - 2, ny); h >= 1; --h) {
       const int ntx = (nx + w - 1) / w, nty = (ny + h - 1) / h;
       const double plane_us = step2_plane_us(bytes, w, h);
       const long long tiles = (long long)ntx * nty;
@@ -133,10 +142,15 @@ Step2Plan step2_plan(int storage, int nx, int ny, int nz, int sms) {
   return best;
 }
 
+Step2Plan step2_plan(int storage, bool force, bool moments, int nx, int ny, int nz, int sms) {
+  return force || moments ? plan_for<SlimBlock>(storage, nx, ny, nz, sms)
+                          : plan_for<WideBlock>(storage, nx, ny, nz, sms);
+}
+
 template <int S, bool WALLS, bool FORCE, bool MOM>
 static cudaError_t launch2(const StepArgs &a, const Moments2 &m, const Step2Plan &p,
                            cudaStream_t s) {
-  const size_t smem = step2_smem<Wide>(S, WALLS);
+  const size_t smem = step2_smem<BlockOf<FORCE, MOM>>(S, WALLS);
   if (p.w == 0)  // the plan's preparation: allow this much shared memory
     return cudaFuncSetAttribute(k_step2<S, WALLS, FORCE, MOM>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -160,10 +174,10 @@ static cudaError_t launch2(const StepArgs &a, const Moments2 &m, const Step2Plan
   b.dom.walls = a.walls;
   b.dom.omega = a.omega;
   b.dom.kf = a.kf;
-  b.consts = pair_consts(a.omega);
+  b.consts = pair_consts(a.omega, a.kf);
   b.plan = p;
   k_step2<S, WALLS, FORCE, MOM>
-      <<<p.ntx * p.nty * p.chunks, Wide::kThreads, smem, s>>>(b);
+      <<<p.ntx * p.nty * p.chunks, BlockOf<FORCE, MOM>::kThreads, smem, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -212,7 +226,8 @@ cudaError_t launch_step2_mom(const StepArgs &a, const Moments2 &m, const Step2Pl
 // Where two steps per launch are faster than two launches of the two-node
 // kernel. FP32: from 400,000 nodes on, where the lattice outgrows L2
 // (measured cavity, two launches against one: 96^3 19.8 / 15.9 us a step,
-// 72^3 9.0 / 10.1, 101 x 67 x 45 7.0 / 8.9, 78 x 237 x 27 11.2 / 9.9). 16-bit
+// 72^3 9.0 / 10.1, 101 x 67 x 45 7.0 / 8.9, 78 x 237 x 27 11.2 / 9.9; with a
+// body force 80^3 14.8 / 12.5, 72^3 11.6 / 12.3). 16-bit
 // storage: only where the two-node kernel's 128-node blocks fit the rows
 // badly (FP16 cavity, 45 x 234 x 328 74.7 / 59.2, 86 x 194 x 115 39.3 / 35.4,
 // 193 x 160 x 129 67.2 / 71.4). Rows of up to 30 nodes leave three quarters

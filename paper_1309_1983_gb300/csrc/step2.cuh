@@ -344,8 +344,20 @@ __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ r
     });
   };
 
+  // body force on the thread's two nodes in plane za - 1 + k
+  auto push_force = [&](int k, P2 (&F)[3]) {
+    const int zr = za - 1 + k;
+    if (t >= half1 || (wz && (zr < 0 || zr >= D.nz))) return;
+    const uint32_t zc = (uint32_t)(zr < 0 ? zr + D.nz : zr >= D.nz ? zr - D.nz : zr) * drow;
+    for (int c = 0; c < 3; ++c)
+      F[c] = pk(LBM_LDGN(D.force + c * (size_t)D.cells + (zc + A.fc)),
+                LBM_LDGN(D.force + c * (size_t)D.cells + (zc + B.fc)));
+  };
+
   RawPair<S> next[Q] = {};  // the next plane's pulled values, in flight meanwhile
+  P2 Fnext[3] = {};
   pull(0, next);
+  if constexpr (FORCE) push_force(0, Fnext);
   int sp = 0, sz = 0, sm = 0;  // k modulo the number of slots, per class
   for (int k = 0; k < planes; ++k) {
     const int zr = za - 1 + k;
@@ -358,16 +370,14 @@ __device__ __forceinline__ void step2_first(typename Store<S>::T *__restrict__ r
       d[i] = as_pair<S>(next[i]);
       if constexpr (FACES != 0 && kEz[i] == -1) d[i] = d[i] + pk(top ? lidc[i] : 0.0f);
     });
-    if (k + 1 < planes) pull(k + 1, next);
+    const P2 F[3] = {Fnext[0], Fnext[1], Fnext[2]};
+    if (k + 1 < planes) {
+      pull(k + 1, next);
+      if constexpr (FORCE) push_force(k + 1, Fnext);
+    }
     if (exists) {
       P2 rho, ux, uy, uz;
-      if constexpr (FORCE) {
-        const uint32_t ca = (uint32_t)z * drow + A.fc;
-        const uint32_t cb = (uint32_t)z * drow + B.fc;
-        collide_pair_force(d, D.omega, D.kf, D.force, D.cells, ca, cb, rho, ux, uy, uz);
-      } else {
-        collide_pair(d, C, rho, ux, uy, uz);
-      }
+      collide_pair<FORCE>(d, C, F, rho, ux, uy, uz);
       if constexpr (MOM) {
         const uint32_t zc = (uint32_t)z * drow;
         const bool out = k >= 1 && k <= zb - za;  // not the planes of the rim
@@ -420,6 +430,17 @@ __device__ __forceinline__ void step2_second(const typename Store<S>::T *__restr
   }
   const uint32_t any = WALLS ? __reduce_or_sync(0xffffffffu, fa | fb) : 0u;
 
+  // body force on the thread's two nodes in plane z, fetched a plane ahead
+  auto force = [&](int z, P2 (&F)[3]) {
+    const uint32_t ca = (uint32_t)z * drow + (uint32_t)(y0 + ya) * D.nx + (x0 + xa);
+    const uint32_t cb = (uint32_t)z * drow + (uint32_t)(y0 + yb) * D.nx + (x0 + xa);
+    for (int c = 0; c < 3; ++c)
+      F[c] = pk(LBM_LDGN(D.force + c * (size_t)D.cells + ca),
+                LBM_LDGN(D.force + c * (size_t)D.cells + cb));
+  };
+  P2 Fnext[3] = {};
+  if constexpr (FORCE) force(za, Fnext);
+
   // plane za - 1 + j of the first step is in slots j modulo (4, 3, 2 or 3);
   // the output plane za - 1 + j pulls from j - 1, j and j + 1
   for (int k = 0; k < 3; ++k) __syncthreads();
@@ -463,13 +484,9 @@ __device__ __forceinline__ void step2_second(const typename Store<S>::T *__restr
         d[i] = pk(da[i], db[i]);
       });
       P2 rho, ux, uy, uz;
-      if constexpr (FORCE) {
-        const uint32_t ca = (uint32_t)z * drow + (uint32_t)(y0 + ya) * D.nx + (x0 + xa);
-        const uint32_t cb = (uint32_t)z * drow + (uint32_t)(y0 + yb) * D.nx + (x0 + xa);
-        collide_pair_force(d, D.omega, D.kf, D.force, D.cells, ca, cb, rho, ux, uy, uz);
-      } else {
-        collide_pair(d, C, rho, ux, uy, uz);
-      }
+      const P2 F[3] = {Fnext[0], Fnext[1], Fnext[2]};
+      if constexpr (FORCE) force(z + 1 < zb ? z + 1 : z, Fnext);
+      collide_pair<FORCE>(d, C, F, rho, ux, uy, uz);
       if constexpr (MOM) {
         const uint32_t zc = (uint32_t)z * drow;
         store_moments(D.rho[1], D.u[1], D.cells, zc + (uint32_t)(y0 + ya) * D.nx + (x0 + xa),
