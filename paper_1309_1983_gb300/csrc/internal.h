@@ -29,6 +29,7 @@ struct StepArgs {
   int onsite;          // 1: walled axes use the on-site velocity rule (onsite.cuh)
   int onsite_lid;      // 1: the top plane's interior moves with lid[] (on-site)
   float lid[3];        // lid velocity u_w
+  int overlap;         // 1: the launch may overlap the end of the kernel before it
 };
 
 // Buffers of a launch over StepArgs, for the LBM_CHECK tables (check.cuh;
@@ -166,6 +167,7 @@ struct BatchArgs {
   const BatchDom *doms;
   const int2 *tiles;  // {domain, first dense node}
   int ntiles, nsteps, parity0, walls_any;
+  int overlap;  // as in StepArgs
   int ndom;
   unsigned *bar_count, *bar_gen;
   int *err;

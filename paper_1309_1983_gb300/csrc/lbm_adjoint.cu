@@ -2,6 +2,7 @@
 // (per-node mathematics in adjoint.cuh): reverse step, loss seed, and the
 // gradient with respect to the initial velocity.
 #include "adjoint.cuh"
+#include "launch.cuh"
 
 namespace lbm {
 
@@ -39,8 +40,9 @@ template <int W, bool FORCE, bool GRADF>
 __global__ void __launch_bounds__(256, LBM_ADJ_MIN_BLOCKS) k_adjoint_step(const AdjArgs a) {
   const StepArgs &g = a.g;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
+  wait_for_previous(y);
   if (x >= g.nx || y >= g.ny) return;
   adjoint_node<(W != 0), FORCE, GRADF>(static_cast<const float *>(g.fin), a.lam_in, a.lam_out,
                                        g.force, a.grad_force, g.nx, g.ny, g.nz, g.pitch,
@@ -54,8 +56,9 @@ template <int W, bool FORCE, bool GRADF>
 __global__ void __launch_bounds__(256) k_adjoint_step_mom(const AdjArgs a) {
   const StepArgs &g = a.g;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
+  wait_for_previous(y);
   if (x >= g.nx || y >= g.ny) return;
   adjoint_node_mom<(W != 0), FORCE, GRADF>(a.rho_n, a.u_n, a.lam_in, a.lam_out, g.force,
                                            a.grad_force, g.nx, g.ny, g.nz, g.pitch, g.plane,
@@ -109,10 +112,9 @@ cudaError_t launch_adjoint_step(const StepArgs &g, const float *lam_in,
   const dim3 grid((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, g.nz), blk(bx, by, 1);
   const int w = g.walls == 0 ? 0 : g.wall_select ? 1 : 2;
   const bool F = g.force != nullptr, G = grad_force != nullptr;
-#define LBM_ADJ_CASE(W_, F_, G_)                                 \
-  if (w == W_ && F == F_ && G == G_) {                           \
-    k_adjoint_step<W_, F_, G_><<<grid, blk, 0, s>>>(a);          \
-    return cudaGetLastError();                                   \
+#define LBM_ADJ_CASE(W_, F_, G_)                                                     \
+  if (w == W_ && F == F_ && G == G_) {                                               \
+    return launch_kernel(g.overlap, k_adjoint_step<W_, F_, G_>, grid, blk, 0, s, a); \
   }
   LBM_ADJ_CASE(0, false, false)
   LBM_ADJ_CASE(0, false, true)
@@ -148,10 +150,9 @@ cudaError_t launch_adjoint_step_mom(const StepArgs &g, const float *rho_n, const
   const dim3 grid((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, g.nz), blk(bx, by, 1);
   const int w = g.walls == 0 ? 0 : g.wall_select ? 1 : 2;
   const bool F = g.force != nullptr, G = grad_force != nullptr;
-#define LBM_ADJ_CASE(W_, F_, G_)                                 \
-  if (w == W_ && F == F_ && G == G_) {                           \
-    k_adjoint_step_mom<W_, F_, G_><<<grid, blk, 0, s>>>(a);      \
-    return cudaGetLastError();                                   \
+#define LBM_ADJ_CASE(W_, F_, G_)                                                     \
+  if (w == W_ && F == F_ && G == G_) {                                               \
+    return launch_kernel(g.overlap, k_adjoint_step_mom<W_, F_, G_>, grid, blk, 0, s, a); \
   }
   LBM_ADJ_CASE(0, false, false)
   LBM_ADJ_CASE(0, false, true)

@@ -12,6 +12,7 @@
 // from shared memory, and the planes are reached by 32-bit offsets from one
 // base: kernel parameters serve neither here.
 #include "internal.h"
+#include "launch.cuh"
 #include "step2.cuh"
 
 namespace lbm {
@@ -25,6 +26,8 @@ __global__ void __launch_bounds__(Slim::kThreads, 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float *ring = reinterpret_cast<float *>(smem_raw);
   __shared__ PairConsts consts;
+  int t = threadIdx.x;
+  wait_for_previous(t);
   const Batch2Item *ip = items + blockIdx.x;
   if (!LBM_VALID(ip)) return;
   const Batch2Item it = *ip;
@@ -47,7 +50,6 @@ __global__ void __launch_bounds__(Slim::kThreads, 1)
   D.walls = B.walls;
   D.omega = B.omega;
   D.kf = B.kf;
-  const int t = threadIdx.x;
   if (t == 0) consts = pair_consts(B.omega, B.kf);
   __syncthreads();
   if (t < Slim::kFirst) {
@@ -82,18 +84,10 @@ cudaError_t launch_batch_step2(const BatchArgs &a, const Batch2Item *items, int 
                   chk_r(fin, LBM_BATCH_F(a)), chk_w(fout, LBM_BATCH_F(a)),
                   chk_w(m.rho[0], LBM_BATCH_FIELD(a, 1)), chk_w(m.u[0], LBM_BATCH_FIELD(a, 3)),
                   chk_w(m.rho[1], LBM_BATCH_FIELD(a, 1)), chk_w(m.u[1], LBM_BATCH_FIELD(a, 3)));
-  if (a.walls_any) {
-    if (m.rho[0])
-      k_batch_step2<true, true><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
-    else
-      k_batch_step2<true, false><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
-  } else {
-    if (m.rho[0])
-      k_batch_step2<false, true><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
-    else
-      k_batch_step2<false, false><<<nitems, Slim::kThreads, smem, s>>>(a, items, fin, fout, m);
-  }
-  return cudaGetLastError();
+  const bool mom = m.rho[0] != nullptr;
+  auto *k = a.walls_any ? (mom ? k_batch_step2<true, true> : k_batch_step2<true, false>)
+                        : (mom ? k_batch_step2<false, true> : k_batch_step2<false, false>);
+  return launch_kernel(a.overlap != 0, k, nitems, Slim::kThreads, smem, s, a, items, fin, fout, m);
 }
 
 }  // namespace lbm

@@ -16,6 +16,7 @@
 
 #include "d3q19.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "tune.h"
 
 using lbm::BatchArgs;
@@ -314,7 +315,8 @@ int persistent_grid(lbm_batch *b, int *grid) {
 // the current buffer: graphs of kGraphPasses while there are enough of them.
 constexpr int kGraphPasses = 16;
 int two_step_passes(lbm_batch *b, int passes) {
-  const BatchArgs a = make_args(b);
+  BatchArgs a = make_args(b);
+  a.overlap = 1;  // lbm_batch_step waits for its launches: no caller captures it
   auto pass = [&](int k, cudaStream_t s) {
     const int c = b->cur ^ (k & 1);
     return lbm::launch_batch_step2(a, b->d_items, b->nitems, b->f[c], b->f[1 - c],
@@ -852,7 +854,8 @@ int lbm_batch_advance(lbm_batch_t *b, int n, const void *f_in, void *f_out, void
     }
     return LBM_OK;
   }
-  const BatchArgs a = make_args(b);
+  BatchArgs a = make_args(b);
+  a.overlap = lbm::may_overlap(b->stream);
   for (int p = 0; p < passes; ++p) {
     const float *fi = static_cast<const float *>(in[p]);
     float *fo = static_cast<float *>(out[p]);

@@ -14,6 +14,7 @@
 
 #include "d3q19.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "step_tma.h"
 
 using lbm::StepArgs;
@@ -95,6 +96,7 @@ StepArgs make_args(const lbm_t *h, const void *fin, void *fout) {
   a.walls = h->flags & (LBM_WALL_X | LBM_WALL_Y | LBM_WALL_Z);
   a.z0 = 0;
   a.zn = h->nz;
+  a.overlap = lbm::may_overlap(h->stream) ? 1 : 0;
   // The one-node kernel with 16-bit storage is issue-bound: there the branch
   // form's shorter common path wins once wall nodes are rare in every warp
   // (long rows). FP32 is bandwidth-bound and the divergence-free select form

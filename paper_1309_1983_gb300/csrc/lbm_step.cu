@@ -13,6 +13,7 @@
 // neighbouring warps still pull.
 #include "d3q19.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "onsite.cuh"
 #include "stream.cuh"
 
@@ -113,8 +114,9 @@ __global__ void __launch_bounds__(kReduceThreads)
   bool bad = false;
   const uint32_t plane_nodes = (uint32_t)a.nx * a.ny;
   const uint32_t dc_end = (uint32_t)(a.z0 + a.zn) * plane_nodes;
-  for (uint32_t dc = (uint32_t)a.z0 * plane_nodes + blockIdx.x * blockDim.x + threadIdx.x;
-       dc < dc_end; dc += gridDim.x * blockDim.x) {
+  int first = (int)((uint32_t)a.z0 * plane_nodes + blockIdx.x * blockDim.x + threadIdx.x);
+  wait_for_previous(first);
+  for (uint32_t dc = (uint32_t)first; dc < dc_end; dc += gridDim.x * blockDim.x) {
     const uint32_t x = dc % a.nx;
     const uint32_t t = dc / a.nx;
     const uint32_t y = t % a.ny, z = t / a.ny;
@@ -237,13 +239,10 @@ cudaError_t launch_init(int storage, const StepArgs &a, const float *rho0,
 }
 
 template <int S>
-static void moments_dispatch(const StepArgs &a, const void *f, float *rho,
-                             float *u, double *partials, int *err, int nb,
-                             cudaStream_t s) {
-  if (a.force)
-    k_moments<S, true><<<nb, kReduceThreads, 0, s>>>(a, f, rho, u, partials, err);
-  else
-    k_moments<S, false><<<nb, kReduceThreads, 0, s>>>(a, f, rho, u, partials, err);
+static cudaError_t moments_dispatch(const StepArgs &a, const void *f, float *rho, float *u,
+                                    double *partials, int *err, int nb, cudaStream_t s) {
+  return launch_kernel(a.overlap, a.force ? k_moments<S, true> : k_moments<S, false>, nb,
+                       kReduceThreads, 0, s, a, f, rho, u, partials, err);
 }
 
 cudaError_t launch_moments(int storage, const StepArgs &a, const void *f,
@@ -261,12 +260,11 @@ cudaError_t launch_moments(int storage, const StepArgs &a, const void *f,
                   chk_r(a.force, 3 * (size_t)a.cells * sizeof(float)),
                   chk_w(partials, (size_t)nb * sizeof(double)), chk_rw(err, sizeof(int)));
   switch (storage) {
-    case kF32: moments_dispatch<0>(a, f, rho, u, partials, err, nb, s); break;
-    case kF16: moments_dispatch<1>(a, f, rho, u, partials, err, nb, s); break;
-    case kBF16: moments_dispatch<2>(a, f, rho, u, partials, err, nb, s); break;
+    case kF32: return moments_dispatch<0>(a, f, rho, u, partials, err, nb, s);
+    case kF16: return moments_dispatch<1>(a, f, rho, u, partials, err, nb, s);
+    case kBF16: return moments_dispatch<2>(a, f, rho, u, partials, err, nb, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 int moments_blocks(uint32_t cells) {

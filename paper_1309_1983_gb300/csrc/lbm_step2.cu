@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "launch.cuh"
 #include "step2.cuh"
 
 namespace lbm {
@@ -65,7 +66,8 @@ __global__ void __launch_bounds__(BlockOf<FORCE, MOM>::kThreads, 1)
   const int za = (int)((long long)D.nz * chunk / p.chunks);
   const int zb = (int)((long long)D.nz * (chunk + 1) / p.chunks);
   const int cw = min(p.w, D.nx - x0), ch = min(p.h, D.ny - y0);
-  const int t = threadIdx.x;
+  int t = threadIdx.x;
+  wait_for_previous(t);
   if (t < Block::kFirst) {
     // a tile away from the x and y walls takes the shorter form
     const bool side = WALLS && (((D.walls & LBM_WALL_X) && (x0 <= 1 || x0 + cw >= D.nx - 1)) ||
@@ -176,9 +178,8 @@ static cudaError_t launch2(const StepArgs &a, const Moments2 &m, const Step2Plan
   b.dom.kf = a.kf;
   b.consts = pair_consts(a.omega, a.kf);
   b.plan = p;
-  k_step2<S, WALLS, FORCE, MOM>
-      <<<p.ntx * p.nty * p.chunks, BlockOf<FORCE, MOM>::kThreads, smem, s>>>(b);
-  return cudaGetLastError();
+  return launch_kernel(a.overlap, k_step2<S, WALLS, FORCE, MOM>, p.ntx * p.nty * p.chunks,
+                       BlockOf<FORCE, MOM>::kThreads, smem, s, b);
 }
 
 static cudaError_t dispatch2(int storage, const StepArgs &a, const Moments2 &m, bool mom,

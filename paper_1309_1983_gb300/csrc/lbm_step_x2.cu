@@ -25,6 +25,7 @@
 
 #include "d3q19.cuh"
 #include "internal.h"
+#include "launch.cuh"
 #include "onsite.cuh"
 #include "pack.cuh"
 #include "stream.cuh"
@@ -141,8 +142,9 @@ template <int S, int W, bool FORCE, bool MOM>
 __global__ void LBM_X2_BOUNDS k_step_x2(const StepArgs a) {
   using T = typename Store<S>::T;
   const int x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = a.z0 + blockIdx.z;
+  wait_for_previous(y);
   if (x0 >= a.nx || y >= a.ny) return;
   const bool has1 = x0 + 1 < a.nx;
   const T *__restrict__ fin = static_cast<const T *>(a.fin);
@@ -224,13 +226,12 @@ __global__ void LBM_X2_BOUNDS k_step_x2(const StepArgs a) {
 }
 
 template <int S>
-static void x2_dispatch(bool moments, const StepArgs &a, dim3 g, dim3 b, cudaStream_t s) {
+static cudaError_t x2_dispatch(bool moments, const StepArgs &a, dim3 g, dim3 b, cudaStream_t s) {
   const int walls = a.walls == 0 ? 0 : a.onsite ? 3 : a.wall_select ? 1 : 2;
   const bool force = a.force != nullptr;
-#define LBM_X2_CASE(W, F, M)                                    \
-  if (walls == W && force == F && moments == M) {               \
-    k_step_x2<S, W, F, M><<<g, b, 0, s>>>(a);                   \
-    return;                                                     \
+#define LBM_X2_CASE(W, F, M)                                               \
+  if (walls == W && force == F && moments == M) {                          \
+    return launch_kernel(a.overlap, k_step_x2<S, W, F, M>, g, b, 0, s, a); \
   }
   LBM_X2_CASE(0, false, false)
   LBM_X2_CASE(0, false, true)
@@ -249,6 +250,7 @@ static void x2_dispatch(bool moments, const StepArgs &a, dim3 g, dim3 b, cudaStr
   LBM_X2_CASE(3, true, false)
   LBM_X2_CASE(3, true, true)
 #undef LBM_X2_CASE
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &a, int bxp, int by,
@@ -257,12 +259,11 @@ cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &a, int bxp
   const dim3 g((pairs + bxp - 1) / bxp, (a.ny + by - 1) / by, a.zn), b(bxp, by, 1);
   LBM_CHECK_TABLE(s, LBM_STEP_RANGES(a, elem_bytes_of(storage)));
   switch (storage) {
-    case kF32: x2_dispatch<0>(moments, a, g, b, s); break;
-    case kF16: x2_dispatch<1>(moments, a, g, b, s); break;
-    case kBF16: x2_dispatch<2>(moments, a, g, b, s); break;
+    case kF32: return x2_dispatch<0>(moments, a, g, b, s);
+    case kF16: return x2_dispatch<1>(moments, a, g, b, s);
+    case kBF16: return x2_dispatch<2>(moments, a, g, b, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace lbm
