@@ -222,7 +222,8 @@ int lbm_set_kernel(lbm_t *h, int variant);
  * steps that write rho and u take one launch each. Results are identical.
  * After such a call the other buffer of the pair holds an earlier state, not
  * always the one before the last step. LBM_FUSE_AUTO (default): for the
- * lattices that it is faster for (FP32 from 400,000 nodes on, and short rows);
+ * lattices that it is faster for (FP32 from 500,000 nodes on, 600,000 with a body force, and
+ * large 16-bit lattices of short rows);
  * LBM_FUSE_OFF: never; LBM_FUSE_ALWAYS: whenever the kernel and the walls
  * allow it. Returns LBM_EINVAL for any other mode. */
 #define LBM_FUSE_AUTO 0
@@ -256,7 +257,8 @@ int lbm_set_graph_steps(lbm_t *h, int steps);
 
 /* Block shape of the pair kernel: bxp pairs along x (a multiple of 32) by
  * `by` rows, bxp * by <= 256, used by LBM_KERNEL_PAIR and LBM_KERNEL_X2
- * (the default kernel). Default: 64 x 2 (1 row when ny = 1). */
+ * (the default kernel). Default: 64 x 2 (1 row when ny = 1), except that
+ * LBM_KERNEL_X2 then lays short rows out in one run where that is faster. */
 int lbm_set_pair_block(lbm_t *h, int bxp, int by);
 
 /* Launch-shape autotuner (no counterpart in the paper, which fixed its block

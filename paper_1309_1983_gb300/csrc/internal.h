@@ -29,6 +29,8 @@ struct StepArgs {
   int onsite;          // 1: walled axes use the on-site velocity rule (onsite.cuh)
   int onsite_lid;      // 1: the top plane's interior moves with lid[] (on-site)
   float lid[3];        // lid velocity u_w
+  // two-node kernel: pairs of a row and 2^32 over it if a plane is one run (else 0)
+  uint32_t flat_pairs, flat_inv;
   int overlap;         // 1: the launch may overlap the end of the kernel before it
 };
 
@@ -64,9 +66,10 @@ cudaError_t launch_step(int storage, bool moments, const StepArgs &a, int bx,
 // 16-bit storage, two x-adjacent nodes per thread (bxp pairs per block row,
 // a multiple of 32).
 // 16-bit storage, two x-adjacent nodes per thread without exchange between
-// threads (bxp pairs per block row, `by` rows).
+// threads (bxp pairs per block row, `by` rows; any_shape: unless another
+// arrangement is faster).
 cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &a, int bxp, int by,
-                           cudaStream_t s);
+                           bool any_shape, cudaStream_t s);
 // Two steps per launch (step2.cuh): tiles of w x h columns, ntx x nty of
 // them, the planes cut into `chunks` runs.
 struct Step2Plan {
@@ -74,7 +77,7 @@ struct Step2Plan {
   float us;  // modelled time of a pass
 };
 // Whether multi-step calls of this lattice are faster so.
-bool step2_wins(int storage, int nx, int ny, int nz);
+bool step2_wins(int storage, bool force, int nx, int ny, int nz);
 // Once per handle and device before its launches.
 cudaError_t prepare_step2(int storage, const StepArgs &a, bool moments);
 Step2Plan step2_plan(int storage, bool force, bool moments, int nx, int ny, int nz, int sms);
@@ -268,6 +271,7 @@ struct lbm_lattice {
   // tiles of the two-step kernel, without and with moments (w = 0: not made yet)
   lbm::Step2Plan plan2[2];
   int pbx, pby;  // block shape of the pair kernel (pairs along x, rows)
+  bool pair_block_set;  // by lbm_set_pair_block (or the autotuner)
   int device;
   lbm::Scratch scr;
   // lbm_run_host pipeline (created on first use, released by lbm_destroy)

@@ -167,7 +167,7 @@ cudaError_t launch_one_step(const lbm_t *h, bool mom, const StepArgs &a, cudaStr
   if (h->kernel == LBM_KERNEL_PAIR && h->storage != lbm::kF32)
     return lbm::launch_step_pair16(h->storage, mom, a, h->pbx, h->pby, s);
   if (h->kernel == LBM_KERNEL_X2)
-    return lbm::launch_step_x2(h->storage, mom, a, h->pbx, h->pby, s);
+    return lbm::launch_step_x2(h->storage, mom, a, h->pbx, h->pby, !h->pair_block_set, s);
   if (h->kernel == LBM_KERNEL_X4)
     return lbm::launch_step_x4(h->storage, mom, a, h->pbx, h->pby, s);
   if (h->kernel == LBM_KERNEL_TMA)
@@ -184,7 +184,8 @@ cudaError_t launch_one_step(const lbm_t *h, bool mom, const StepArgs &a) {
 // Whether multi-step calls advance two steps per launch.
 bool fuses(const lbm_t *h) {
   if (h->kernel != LBM_KERNEL_X2 || onsite(h) || h->fuse == LBM_FUSE_OFF) return false;
-  return h->fuse == LBM_FUSE_ALWAYS || lbm::step2_wins(h->storage, h->nx, h->ny, h->nz);
+  return h->fuse == LBM_FUSE_ALWAYS ||
+         lbm::step2_wins(h->storage, (h->flags & LBM_FORCE) != 0, h->nx, h->ny, h->nz);
 }
 
 // The two-step kernel's tiles, made before the first launch that needs them.
@@ -441,6 +442,7 @@ int lbm_create(int nx, int ny, int nz, float tau, uint32_t flags,
   h->wall_mode = LBM_WALLS_AUTO;
   h->pbx = 64;  // 64 pairs x 2 rows measured best for the two-node kernel
   h->pby = ny < 2 ? ny : 2;
+  h->pair_block_set = false;
   h->device = -1;
   h->stage = nullptr;
   h->pipe_ready = false;
@@ -596,6 +598,7 @@ int lbm_set_pair_block(lbm_t *h, int bxp, int by) {
     return fail(LBM_EINVAL, "pair block must be bxp%32==0, by>=1, bxp*by<=256");
   h->pbx = bxp;
   h->pby = by;
+  h->pair_block_set = true;
   h->config_version++;
   return LBM_OK;
 }

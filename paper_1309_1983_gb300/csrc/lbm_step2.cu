@@ -225,20 +225,17 @@ cudaError_t launch_step2_mom(const StepArgs &a, const Moments2 &m, const Step2Pl
 }
 
 // Where two steps per launch are faster than two launches of the two-node
-// kernel. FP32: from 400,000 nodes on, where the lattice outgrows L2
-// (measured cavity, two launches against one: 96^3 19.8 / 15.9 us a step,
-// 72^3 9.0 / 10.1, 101 x 67 x 45 7.0 / 8.9, 78 x 237 x 27 11.2 / 9.9; with a
-// body force 80^3 14.8 / 12.5, 72^3 11.6 / 12.3). 16-bit
-// storage: only where the two-node kernel's 128-node blocks fit the rows
-// badly (FP16 cavity, 45 x 234 x 328 74.7 / 59.2, 86 x 194 x 115 39.3 / 35.4,
-// 193 x 160 x 129 67.2 / 71.4). Rows of up to 30 nodes leave three quarters
-// of its threads idle, and two steps per launch win from 60,000 nodes on
-// (24 x 200 x 24 5.7 / 4.7, 20 x 60 x 60 4.6 / 4.4).
-bool step2_wins(int storage, int nx, int ny, int nz) {
+// kernel. FP32: from where the lattice outgrows L2 (measured cavity, two
+// launches against one, us a step: 96^3 18.2 / 15.7, 78 x 237 x 27 10.1 / 9.7,
+// 72^3 7.3 / 10.2, 101 x 67 x 45 6.6 / 8.7; with a body force 96^3 28.1 / 22.2,
+// 101 x 67 x 85 17.1 / 16.3). 16-bit storage: only on short rows that start at
+// any offset, which the two-node kernel's loads suit least (FP16 cavity,
+// 45 x 234 x 328 71.2 / 58.5, 86 x 194 x 115 39.1 / 34.8; 160^3 55.6 / 69.3,
+// 78 x 237 x 27 7.5 / 10.0, 193 x 160 x 129 67.1 / 70.4).
+bool step2_wins(int storage, bool force, int nx, int ny, int nz) {
   const double nodes = (double)nx * ny * nz;
-  if (nx <= 30) return nodes >= 6e4;
-  if (nodes < 4e5) return false;
-  return storage == kF32 || nx < 0.7 * 128 * ((nx + 127) / 128);
+  if (storage == kF32) return nodes >= (force ? 6e5 : 5e5);
+  return nx <= 90 && nx % 16 != 0 && nodes >= 1.5e6;
 }
 
 }  // namespace lbm

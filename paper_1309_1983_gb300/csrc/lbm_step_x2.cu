@@ -138,11 +138,26 @@ __device__ __forceinline__ void pull_pair_xwall(const typename Store<S>::T *__re
 // the wall-node branch (the one-node kernel's face fix-ups, per node of the
 // pair), 3 on-site velocity walls (plain pulls, then the rule of onsite.cuh
 // on each wall node of the pair).
-template <int S, int W, bool FORCE, bool MOM>
+// FLAT: the pairs of a plane in one run over the blocks (see x2_flat), else
+// blocks of pairs along x by rows.
+template <int S, int W, bool FORCE, bool MOM, bool FLAT>
 __global__ void LBM_X2_BOUNDS k_step_x2(const StepArgs a) {
   using T = typename Store<S>::T;
-  const int x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  int y = blockIdx.y * blockDim.y + threadIdx.y;
+  int x0, y;
+  if constexpr (FLAT) {
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x, p = a.flat_pairs;
+    uint32_t q = __umulhi(k, a.flat_inv);  // k / p or one less
+    uint32_t r = k - q * p;
+    if (r >= p) {
+      r -= p;
+      ++q;
+    }
+    x0 = 2 * (int)r;
+    y = (int)q;
+  } else {
+    x0 = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+  }
   const int z = a.z0 + blockIdx.z;
   wait_for_previous(y);
   if (x0 >= a.nx || y >= a.ny) return;
@@ -226,42 +241,72 @@ __global__ void LBM_X2_BOUNDS k_step_x2(const StepArgs a) {
 }
 
 template <int S>
-static cudaError_t x2_dispatch(bool moments, const StepArgs &a, dim3 g, dim3 b, cudaStream_t s) {
-  const int walls = a.walls == 0 ? 0 : a.onsite ? 3 : a.wall_select ? 1 : 2;
-  const bool force = a.force != nullptr;
-#define LBM_X2_CASE(W, F, M)                                               \
-  if (walls == W && force == F && moments == M) {                          \
-    return launch_kernel(a.overlap, k_step_x2<S, W, F, M>, g, b, 0, s, a); \
-  }
-  LBM_X2_CASE(0, false, false)
-  LBM_X2_CASE(0, false, true)
-  LBM_X2_CASE(0, true, false)
-  LBM_X2_CASE(0, true, true)
-  LBM_X2_CASE(1, false, false)
-  LBM_X2_CASE(1, false, true)
-  LBM_X2_CASE(1, true, false)
-  LBM_X2_CASE(1, true, true)
-  LBM_X2_CASE(2, false, false)
-  LBM_X2_CASE(2, false, true)
-  LBM_X2_CASE(2, true, false)
-  LBM_X2_CASE(2, true, true)
-  LBM_X2_CASE(3, false, false)
-  LBM_X2_CASE(3, false, true)
-  LBM_X2_CASE(3, true, false)
-  LBM_X2_CASE(3, true, true)
+static cudaError_t x2_dispatch(bool moments, int walls, const StepArgs &a, dim3 g, dim3 b,
+                               cudaStream_t s) {
+  const bool force = a.force != nullptr, flat = a.flat_pairs != 0;
+#define LBM_X2_CASE(W, F, M, L)                                               \
+  if (walls == W && force == F && moments == M && flat == L)                  \
+    return launch_kernel(a.overlap, k_step_x2<S, W, F, M, L>, g, b, 0, s, a);
+#define LBM_X2_CASES(W, L)        \
+  LBM_X2_CASE(W, false, false, L) \
+  LBM_X2_CASE(W, false, true, L)  \
+  LBM_X2_CASE(W, true, false, L)  \
+  LBM_X2_CASE(W, true, true, L)
+  LBM_X2_CASES(0, false)
+  LBM_X2_CASES(1, false)
+  LBM_X2_CASES(2, false)
+  LBM_X2_CASES(3, false)
+  LBM_X2_CASES(0, true)
+  LBM_X2_CASES(1, true)
+  LBM_X2_CASES(3, true)
+#undef LBM_X2_CASES
 #undef LBM_X2_CASE
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &a, int bxp, int by,
-                           cudaStream_t s) {
+// Whether the pairs of a plane go to the threads in one run over all rows,
+// with a division per thread, instead of blocks of 64 pairs x 2 rows, where
+// `full` is the share of the lanes that a row's warps fill. Measured, us a
+// step, blocks / run: cavity FP32 12 x 100 x 200 16.3 / 6.7, 48^3 3.8 / 3.0,
+// 72^3 8.7 / 6.9, 96^3 19.9 / 18.5, but 64^3 periodic (full warps) 5.1 / 5.3
+// and 101 x 67 x 45 with force 7.5 / 8.0; FP16, bound by instructions, gains
+// on fuller warps too: 96^3 15.1 / 11.8, 101 x 67 x 45 6.1 / 5.3, 112^3
+// 20.6 / 19.2. On longer rows the run's warps straddle them at any offset
+// (FP16 193 x 160 x 129 70.8 / 73.3, 300^3 395 / 416), which costs nothing
+// only without padding: 160 x 160 x 40 FP32 24.0 / 22.9, FP16 16.1 / 13.4.
+// On-site walls: warps of several rows hold more wall nodes (BF16 96^3
+// 18.2 / 16.2, 120 x 120 x 60 15.2 / 16.9). Lattices of a few blocks gain
+// nothing from full ones.
+static bool x2_flat(int storage, const StepArgs &a, int walls) {
   const int pairs = (a.nx + 1) / 2;
-  const dim3 g((pairs + bxp - 1) / bxp, (a.ny + by - 1) / by, a.zn), b(bxp, by, 1);
+  const double full = (double)pairs / ((pairs + 31) / 32 * 32);
+  if (walls == 2 || (long long)pairs * a.ny * a.zn < 4096) return false;
+  if (walls == 3) return a.nx <= 128 && pairs < 58;
+  if (a.nx <= 128) return storage == kF32 ? full < 0.78 : pairs < 64;
+  return full < 0.9 && a.nx % (32 / elem_bytes_of(storage)) == 0;
+}
+
+cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &args, int bxp, int by,
+                           bool any_shape, cudaStream_t s) {
+  const int pairs = (args.nx + 1) / 2;
+  const int walls = args.walls == 0 ? 0 : args.onsite ? 3 : args.wall_select ? 1 : 2;
+  dim3 g((pairs + bxp - 1) / bxp, (args.ny + by - 1) / by, args.zn), b(bxp, by, 1);
+  StepArgs a = args;
+  a.flat_pairs = 0;
+  if (any_shape && x2_flat(storage, a, walls)) {
+    const long long plane = (long long)pairs * a.ny;
+    a.flat_pairs = (uint32_t)pairs;
+    a.flat_inv = pairs == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / pairs);
+    // 64: lattices of a few blocks per SM share them out more evenly (72^3 FP32
+    // 6.9 / 7.3 us with 128), and larger ones do not care
+    b = dim3(64, 1, 1);
+    g = dim3((unsigned)((plane + 63) / 64), 1, a.zn);
+  }
   LBM_CHECK_TABLE(s, LBM_STEP_RANGES(a, elem_bytes_of(storage)));
   switch (storage) {
-    case kF32: return x2_dispatch<0>(moments, a, g, b, s);
-    case kF16: return x2_dispatch<1>(moments, a, g, b, s);
-    case kBF16: return x2_dispatch<2>(moments, a, g, b, s);
+    case kF32: return x2_dispatch<0>(moments, walls, a, g, b, s);
+    case kF16: return x2_dispatch<1>(moments, walls, a, g, b, s);
+    case kBF16: return x2_dispatch<2>(moments, walls, a, g, b, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -65,7 +65,7 @@ def test_default_takes_it_for_large_lattices():
     plain launches and a last step that writes rho and u; and inside a stream
     capture of the caller's."""
     from paper_1309_1983_gb300.lattice import Lattice
-    dims = (83, 81, 67)  # 450,441 nodes
+    dims = (83, 81, 79)  # 531,117 nodes
     u = torch.from_numpy(W.noise((3,) + dims[::-1], 5, 0.04)).float().cuda()
     outs = []
     for mode in ("off", "auto"):
