@@ -258,7 +258,7 @@ int lbm_set_graph_steps(lbm_t *h, int steps);
 /* Block shape of the pair kernel: bxp pairs along x (a multiple of 32) by
  * `by` rows, bxp * by <= 256, used by LBM_KERNEL_PAIR and LBM_KERNEL_X2
  * (the default kernel). Default: 64 x 2 (1 row when ny = 1), except that
- * LBM_KERNEL_X2 then lays short rows out in one run where that is faster. */
+ * LBM_KERNEL_X2 then lays a plane out in one run where that is faster. */
 int lbm_set_pair_block(lbm_t *h, int bxp, int by);
 
 /* Launch-shape autotuner (no counterpart in the paper, which fixed its block

@@ -29,7 +29,7 @@ struct StepArgs {
   int onsite;          // 1: walled axes use the on-site velocity rule (onsite.cuh)
   int onsite_lid;      // 1: the top plane's interior moves with lid[] (on-site)
   float lid[3];        // lid velocity u_w
-  // two-node kernel: pairs of a row and 2^32 over it if a plane is one run (else 0)
+  // two-node kernel: pairs of a padded row and 2^32 over it if a plane is one run (else 0)
   uint32_t flat_pairs, flat_inv;
   int overlap;         // 1: the launch may overlap the end of the kernel before it
 };

@@ -138,7 +138,7 @@ __device__ __forceinline__ void pull_pair_xwall(const typename Store<S>::T *__re
 // the wall-node branch (the one-node kernel's face fix-ups, per node of the
 // pair), 3 on-site velocity walls (plain pulls, then the rule of onsite.cuh
 // on each wall node of the pair).
-// FLAT: the pairs of a plane in one run over the blocks (see x2_flat), else
+// FLAT: the pairs of a plane in one run over the blocks (x2_flat), else
 // blocks of pairs along x by rows.
 template <int S, int W, bool FORCE, bool MOM, bool FLAT>
 __global__ void LBM_X2_BOUNDS k_step_x2(const StepArgs a) {
@@ -264,26 +264,22 @@ static cudaError_t x2_dispatch(bool moments, int walls, const StepArgs &a, dim3 
   return cudaErrorInvalidValue;
 }
 
-// Whether the pairs of a plane go to the threads in one run over all rows,
-// with a division per thread, instead of blocks of 64 pairs x 2 rows, where
-// `full` is the share of the lanes that a row's warps fill. Measured, us a
-// step, blocks / run: cavity FP32 12 x 100 x 200 16.3 / 6.7, 48^3 3.8 / 3.0,
-// 72^3 8.7 / 6.9, 96^3 19.9 / 18.5, but 64^3 periodic (full warps) 5.1 / 5.3
-// and 101 x 67 x 45 with force 7.5 / 8.0; FP16, bound by instructions, gains
-// on fuller warps too: 96^3 15.1 / 11.8, 101 x 67 x 45 6.1 / 5.3, 112^3
-// 20.6 / 19.2. On longer rows the run's warps straddle them at any offset
-// (FP16 193 x 160 x 129 70.8 / 73.3, 300^3 395 / 416), which costs nothing
-// only without padding: 160 x 160 x 40 FP32 24.0 / 22.9, FP16 16.1 / 13.4.
-// On-site walls: warps of several rows hold more wall nodes (BF16 96^3
-// 18.2 / 16.2, 120 x 120 x 60 15.2 / 16.9). Lattices of a few blocks gain
-// nothing from full ones.
-static bool x2_flat(int storage, const StepArgs &a, int walls) {
+// Whether the pairs of a plane go to the threads in one run over its padded
+// rows, with a division per thread, instead of blocks of 64 pairs x 2 rows.
+// A run keeps every warp's accesses on the same lines as the plane itself and
+// leaves only the padding's lanes idle; blocks leave up to 31 of 32. Measured,
+// us a step, blocks / run: cavity FP32 20 x 60 x 60 4.4 / 3.1, 48^3 3.8 / 3.0,
+// 72^3 8.8 / 7.1, 131 x 100 x 100 36.6 / 34.4, 300^3 620.5 / 619.4; FP16 72^3
+// 9.2 / 6.4, 96^3 15.1 / 11.7, 193 x 160 x 129 66.9 / 62.6, 300^3 372 / 368;
+// on-site BF16 193 x 160 x 129 71.1 / 63.8. Where a row fills its warps the
+// division only costs: periodic FP32 64^3 5.1 / 5.3, cavity FP16 320 x 200 x 100
+// 82.0 / 84.3 (on-site walls, which diverge less so, still gain there: 86.8 /
+// 84.8), 384^3 689 / 691. Lattices of a few blocks gain nothing either way.
+static bool x2_flat(const StepArgs &a, int walls) {
   const int pairs = (a.nx + 1) / 2;
-  const double full = (double)pairs / ((pairs + 31) / 32 * 32);
   if (walls == 2 || (long long)pairs * a.ny * a.zn < 4096) return false;
-  if (walls == 3) return a.nx <= 128 && pairs < 58;
-  if (a.nx <= 128) return storage == kF32 ? full < 0.78 : pairs < 64;
-  return full < 0.9 && a.nx % (32 / elem_bytes_of(storage)) == 0;
+  if (walls == 3) return pairs % 64 != 0;
+  return pairs < 0.95 * ((pairs + 31) / 32 * 32);
 }
 
 cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &args, int bxp, int by,
@@ -293,10 +289,11 @@ cudaError_t launch_step_x2(int storage, bool moments, const StepArgs &args, int 
   dim3 g((pairs + bxp - 1) / bxp, (args.ny + by - 1) / by, args.zn), b(bxp, by, 1);
   StepArgs a = args;
   a.flat_pairs = 0;
-  if (any_shape && x2_flat(storage, a, walls)) {
-    const long long plane = (long long)pairs * a.ny;
-    a.flat_pairs = (uint32_t)pairs;
-    a.flat_inv = pairs == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / pairs);
+  if (any_shape && x2_flat(a, walls)) {
+    const int row = a.pitch / 2;
+    const long long plane = (long long)row * a.ny;
+    a.flat_pairs = (uint32_t)row;
+    a.flat_inv = (uint32_t)((1ull << 32) / row);
     // 64: lattices of a few blocks per SM share them out more evenly (72^3 FP32
     // 6.9 / 7.3 us with 128), and larger ones do not care
     b = dim3(64, 1, 1);

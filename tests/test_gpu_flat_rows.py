@@ -1,5 +1,5 @@
 """The two-node kernel with the pairs of a plane in one run over the blocks
-(its default for short rows) against blocks of 64 pairs x 2 rows: the same
+(its default where rows fill their warps badly) against blocks of 64 pairs x 2 rows: the same
 bits, on rows of one node, of odd lengths, around a warp and a block, and on
 longer rows without padding."""
 
@@ -22,7 +22,7 @@ GEOMS = {"periodic": ((0, 0, 0), None, False), "walls_y": ((0, 1, 0), None, Fals
          "cavity": ((1, 1, 1), (0.05, 0.01, 0.0), False),
          "onsite": ((1, 1, 1), (0.05, 0.0, 0.0), True)}
 SHAPES = [(1, 90, 60), (3, 70, 30), (37, 61, 9), (63, 33, 5), (101, 30, 11), (127, 17, 4),
-          (160, 9, 11)]
+          (160, 9, 11), (193, 8, 9), (300, 5, 7)]
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
