@@ -859,11 +859,12 @@ int lbm_run_host(lbm_t *h, const float *u0_host, int n, float *rho_host,
   LBM_CUDA(cudaStreamWaitEvent(h->copy_out, h->ev_start, 0), "stream wait");
   auto copy_in_and_init = [&](int k) -> int {
     if (u0_host) {
+      // one strided copy for the three components
       const size_t off = (size_t)zs[k] * nxy, len = (size_t)(zs[k + 1] - zs[k]) * nxy;
-      for (int c = 0; c < 3; ++c)
-        LBM_CUDA(cudaMemcpyAsync(u0d + c * cells + off, u0_host + c * cells + off,
-                                 len * sizeof(float), cudaMemcpyHostToDevice, h->copy_in),
-                 "u0 copy");
+      const size_t stride = cells * sizeof(float);
+      LBM_CUDA(cudaMemcpy2DAsync(u0d + off, stride, u0_host + off, stride, len * sizeof(float), 3,
+                                 cudaMemcpyHostToDevice, h->copy_in),
+               "u0 copy");
     }
     LBM_CUDA(cudaEventRecord(h->ev_in[k], h->copy_in), "event record");
     LBM_CUDA(cudaStreamWaitEvent(h->stream, h->ev_in[k], 0), "stream wait");
@@ -891,10 +892,9 @@ int lbm_run_host(lbm_t *h, const float *u0_host, int n, float *rho_host,
     const size_t off = (size_t)zs[k] * nxy, len = (size_t)(zs[k + 1] - zs[k]) * nxy;
     LBM_CUDA(cudaMemcpyAsync(rho_host + off, rd + off, len * sizeof(float),
                              cudaMemcpyDeviceToHost, h->copy_out), "rho copy");
-    for (int c = 0; c < 3; ++c)
-      LBM_CUDA(cudaMemcpyAsync(u_host + c * cells + off, ud + c * cells + off,
-                               len * sizeof(float), cudaMemcpyDeviceToHost, h->copy_out),
-               "u copy");
+    const size_t stride = cells * sizeof(float);
+    LBM_CUDA(cudaMemcpy2DAsync(u_host + off, stride, ud + off, stride, len * sizeof(float), 3,
+                               cudaMemcpyDeviceToHost, h->copy_out), "u copy");
     return LBM_OK;
   };
   if (n == 1 && S >= 3) {
