@@ -205,11 +205,18 @@ bool pairs_win(const lbm_batch *b) {
 // The items of a two-step pass. Each domain's columns are cut into its best
 // tiles, and the planes of all of them into runs of at most `most`; the value
 // of `most` is the one for which blocks that take the items in order, longest
-// run first, end soonest (a run walks 3 planes more than it writes).
-int upload_items(lbm_batch *b) {
-  if (b->d_items) return LBM_OK;
+// run first, end soonest (a run walks 3 planes more than it writes). More than
+// 6 items per SM were never better (1 to 256 domains of 16 to 96 nodes a side) and
+// cost the first call most: 64 of them 350 us up to 16 an SM, 40 up to 6. False if
+// they cannot be had (no memory): the calls then go on one step at a time.
+bool upload_items(lbm_batch *b) try {
+  if (b->d_items) return true;
+  const bool walls = (b->flags & (LBM_WALL_X | LBM_WALL_Y | LBM_WALL_Z)) != 0;
+  for (int m = 0; m < 2; ++m)
+    if (lbm::prepare_batch_step2(walls, m != 0) != cudaSuccess) return cudaGetLastError(), false;
   int sms = 0;
-  BCUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device), "SM count");
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess)
+    return cudaGetLastError(), false;
   struct Cut {
     int dom, w, h, chunks;
     double us;  // one run of one tile
@@ -232,7 +239,7 @@ int upload_items(lbm_batch *b) {
       cuts.push_back({d, tw[d], th[d], c, tus[d] * ((D.nz + c - 1) / c + 3)});
       n += (size_t)c * ((D.nx + tw[d] - 1) / tw[d]) * ((D.ny + th[d] - 1) / th[d]);
     }
-    if (n > 16 * (size_t)sms && !best.empty()) break;
+    if (n > 6 * (size_t)sms && !best.empty()) break;
     std::stable_sort(cuts.begin(), cuts.end(),
                      [](const Cut &x, const Cut &y) { return x.us > y.us; });
     std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
@@ -265,14 +272,20 @@ int upload_items(lbm_batch *b) {
                            (int)((long long)D.nz * (k + 1) / c.chunks), 0});
   }
   const size_t bytes = items.size() * sizeof(items[0]);
-  BCUDA(cudaMalloc(&b->d_items, bytes), "cudaMalloc items");
-  BCUDA(cudaMemcpy(b->d_items, items.data(), bytes, cudaMemcpyHostToDevice), "item upload");
+  lbm::Batch2Item *p = nullptr;
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e == cudaSuccess) e = cudaMemcpy(p, items.data(), bytes, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(p);
+    return false;
+  }
+  b->d_items = p;
   b->nitems = (int)items.size();
   b->pass_us = best_us;
-  const bool walls = (b->flags & (LBM_WALL_X | LBM_WALL_Y | LBM_WALL_Z)) != 0;
-  for (int m = 0; m < 2; ++m)
-    BCUDA(lbm::prepare_batch_step2(walls, m != 0), "two-step kernel setup");
-  return LBM_OK;
+  return true;
+} catch (const std::bad_alloc &) {
+  return false;
 }
 
 BatchArgs make_args(const lbm_batch *b) {
@@ -577,9 +590,8 @@ int lbm_batch_step(lbm_batch_t *b, int n) {
   if (rc) return rc;
   if (n < 0) return bfail(LBM_EINVAL, "n must be >= 0");
   if (n == 0) return LBM_OK;
-  const bool may_pair = n >= 4 && b->inject_extra == 0 && b->fuse != LBM_FUSE_OFF;
-  if (may_pair && (rc = upload_items(b))) return rc;
-  if (may_pair && pairs_win(b)) {
+  if (n >= 4 && b->inject_extra == 0 && b->fuse != LBM_FUSE_OFF && upload_items(b) &&
+      pairs_win(b)) {
     // groups of four steps as two passes of two, which end in the same buffer
     rc = two_step_passes(b, n / 4 * 2);
     if (rc) return rc;
@@ -833,23 +845,23 @@ int lbm_batch_advance(lbm_batch_t *b, int n, const void *f_in, void *f_out, void
   if ((rho == nullptr) != (u == nullptr)) return bfail(LBM_EINVAL, "give both rho and u or neither");
   for (int k = 0; rho && k < n; ++k)
     if (!rho[k] || !u[k]) return bfail(LBM_EINVAL, "NULL rho or u buffer");
-  bool pair = n >= 2 && b->inject_extra == 0 && b->fuse != LBM_FUSE_OFF;
-  if (pair && (rc = upload_items(b))) return rc;
-  pair = pair && pairs_win(b);
+  const bool pair = n >= 2 && b->inject_extra == 0 && b->fuse != LBM_FUSE_OFF &&
+                    upload_items(b) && pairs_win(b);
   // passes of two steps and a last one of one, or of one step each; they
   // alternate between the two buffers and end in f_out
-  const int per = pair ? 2 : 1;
-  const int passes = (n + per - 1) / per;
-  std::vector<const void *> in(passes);
-  std::vector<void *> out(passes);
-  for (int p = 0; p < passes; ++p) {
-    out[p] = (passes - p) % 2 ? f_out : f_tmp;
-    in[p] = p == 0 ? f_in : out[p - 1];
-  }
+  const int passes = pair ? (n + 1) / 2 : n;
+  auto out = [&](int p) { return (passes - p) % 2 ? f_out : f_tmp; };
+  auto in = [&](int p) { return p == 0 ? f_in : out(p - 1); };
   if (!pair) {
     for (int k = 0; k < n; k += lbm::kMaxSeqSteps) {
       const int m = std::min(lbm::kMaxSeqSteps, n - k);
-      rc = lbm_batch_run(b, m, &in[k], &out[k], rho ? rho + k : nullptr, u ? u + k : nullptr);
+      const void *ins[lbm::kMaxSeqSteps];
+      void *outs[lbm::kMaxSeqSteps];
+      for (int j = 0; j < m; ++j) {
+        ins[j] = in(k + j);
+        outs[j] = out(k + j);
+      }
+      rc = lbm_batch_run(b, m, ins, outs, rho ? rho + k : nullptr, u ? u + k : nullptr);
       if (rc) return rc;
     }
     return LBM_OK;
@@ -857,8 +869,8 @@ int lbm_batch_advance(lbm_batch_t *b, int n, const void *f_in, void *f_out, void
   BatchArgs a = make_args(b);
   a.overlap = lbm::may_overlap(b->stream);
   for (int p = 0; p < passes; ++p) {
-    const float *fi = static_cast<const float *>(in[p]);
-    float *fo = static_cast<float *>(out[p]);
+    const float *fi = static_cast<const float *>(in(p));
+    float *fo = static_cast<float *>(out(p));
     const int k = 2 * p;
     cudaError_t e;
     if (k + 1 < n) {

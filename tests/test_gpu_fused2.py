@@ -2,10 +2,13 @@
 launch of the two-node kernel, at the sizes where a tile, its rim, a chunk of
 planes or a remainder of steps can go wrong."""
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
 
+from paper_1309_1983_gb300 import capi
 from paper_1309_1983_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -97,6 +100,60 @@ def test_default_takes_it_for_large_lattices():
     np.testing.assert_array_equal(L.get_f(), R.get_f())
 
 
+def _ptrs(ts):
+    return (ctypes.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
+
+
+def _advance(entry, handle, n, f0, fields, fuse):
+    """f after n steps of `entry` from f0 and, if `fields` says how many nodes
+    there are, every step's rho and u."""
+    fuse("always" if n > 1 else "off")
+    bufs = [f0] + [torch.zeros_like(f0) for _ in range(2)]
+    rho = [torch.full((fields,), 9.0, device="cuda") for _ in range(n if fields else 0)]
+    u = [torch.full((3 * fields,), 9.0, device="cuda") for _ in range(n if fields else 0)]
+    capi.call(entry, handle, n, *[ctypes.c_void_p(b.data_ptr()) for b in bufs],
+              _ptrs(rho) if fields else None, _ptrs(u) if fields else None)
+    torch.cuda.synchronize()
+    return bufs[1], rho, u
+
+
+def _against_singles(entry, handle, f0, fields, fuse, nodes=lambda f: f):
+    """2 and 5 steps (with a remainder) against as many calls of one step."""
+    for n in (2, 5):
+        keep = f0.clone()
+        f, rho, u = _advance(entry, handle, n, f0, fields, fuse)
+        assert torch.equal(f0, keep)
+        ref = f0
+        for k in range(n):
+            ref, r, v = _advance(entry, handle, 1, ref, fields, fuse)
+            if fields:
+                assert torch.equal(rho[k], r[0]) and torch.equal(u[k], v[0])
+        assert torch.equal(nodes(f), nodes(ref))
+
+
+@pytest.mark.parametrize("force", [False, True])
+@pytest.mark.parametrize("geom", ["periodic", "walls_x", "cavity"])
+@pytest.mark.parametrize("shape", [(1, 7, 6), (37, 11, 9), (70, 45, 33), (50, 33, 2)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_advance_with_and_without_moments(shape, geom, force):
+    from paper_1309_1983_gb300.lattice import Lattice
+    nx, ny, nz = shape
+    walls, lid = GEOMS[geom]
+    L = Lattice(nx, ny, nz, 0.62, walls=tuple(bool(w) for w in walls), lid=lid, force=force)
+    if force:
+        L.force.copy_(torch.from_numpy(W.noise((3, nz, ny, nx), 3, 1e-3)).float())
+    L.init_equilibrium(u=torch.from_numpy(W.noise((3, nz, ny, nx), 2, 0.04)).float().cuda())
+    rows, pitch = ny * nz, -(-nx // 8) * 8  # single steps also write the padding
+
+    def nodes(f):
+        return f.view(torch.float32)[:19 * rows * pitch].view(19, rows, pitch)[..., :nx]
+
+    for fields in (0, nx * ny * nz):
+        _against_singles("lbm_advance", L.handle, L.current_buffers()[0], fields, L.set_fusion,
+                         nodes)
+    L.close()
+
+
 BATCH_DIMS = [(17, 5, 9), (33, 16, 4), (1, 6, 7), (40, 3, 3), (8, 8, 8), (70, 45, 33), (5, 1, 1)]
 
 
@@ -122,3 +179,15 @@ def test_batch_has_the_bits_of_single_steps(walls):
     for d in range(len(BATCH_DIMS)):
         np.testing.assert_array_equal(got[0][0][d], got[1][0][d])
     assert got[0][1] == got[1][1]
+
+
+@pytest.mark.parametrize("walls", [(1, 1, 1), (0, 0, 0)])
+def test_batch_advance_with_and_without_moments(walls):
+    from paper_1309_1983_gb300.batch import Batch
+    B = Batch(BATCH_DIMS, [0.55, 0.7, 0.9, 1.0, 0.62, 0.6, 0.8],
+              [0.02, 0.05, 0.08, 0.03, 0.06, 0.05, 0.04] if walls[2] else None,
+              walls=tuple(bool(w) for w in walls), lid=bool(walls[2]))
+    B.init_equilibrium(torch.from_numpy(W.noise(3 * B.cells, 7, 0.04)).float().cuda())
+    for fields in (0, B.cells):
+        _against_singles("lbm_batch_advance", B.handle, B.current_buffers()[0], fields,
+                         B.set_fusion)
