@@ -40,8 +40,9 @@
  *     x fastest, each x row padded to `pitch` elements (32-byte aligned
  *     rows), element type FP32, FP16 or BF16 per LBM_STORE_*, holding the
  *     SHIFTED value f_i - w_i. Padding elements never enter the result (the
- *     two-node 16-bit kernels load and store the padding element of an odd
- *     row together with the row's last node).
+ *     two-node kernels load and store the padding element of an odd row
+ *     together with the row's last node; two steps per launch write zeros
+ *     into all of a row's padding).
  *   - Field buffers (rho, velocity u, force F, targets, gradients) are dense
  *     FP32 planes without padding: scalars [nz][ny][nx], vectors
  *     [3][nz][ny][nx] (component-major).

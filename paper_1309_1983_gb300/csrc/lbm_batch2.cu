@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(Slim::kThreads, 1)
       step2_first<0, WALLS ? 1 : 0, WALLS, false, MOM, Slim::kCap>(
           ring, D, consts, B.lidc, it.x0, it.y0, it.cw, it.ch, it.za, it.zb, t);
   } else {
-    step2_second<0, WALLS, false, MOM, Slim::kCap>(ring, D, consts, B.lidc, it.x0, it.y0, it.cw,
+    step2_second<0, WALLS, false, MOM, Slim::kCap, Slim::kSecond>(ring, D, consts, B.lidc, it.x0, it.y0, it.cw,
                                                   it.ch, it.za, it.zb, t - Slim::kFirst);
   }
 }

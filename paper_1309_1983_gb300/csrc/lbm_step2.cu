@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(BlockOf<FORCE, MOM>::kThreads, 1)
       step2_first<S, WALLS ? 1 : 0, WALLS, FORCE, MOM, Block::kCap>(ring, D, a.consts, a.lidc, x0,
                                                                   y0, cw, ch, za, zb, t);
   } else {
-    step2_second<S, WALLS, FORCE, MOM, Block::kCap>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za,
+    step2_second<S, WALLS, FORCE, MOM, Block::kCap, Block::kSecond>(ring, D, a.consts, a.lidc, x0, y0, cw, ch, za,
                                                   zb, t - Block::kFirst);
   }
 }
