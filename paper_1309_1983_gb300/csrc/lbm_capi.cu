@@ -181,17 +181,27 @@ cudaError_t launch_one_step(const lbm_t *h, bool mom, const StepArgs &a) {
   return launch_one_step(h, mom, a, h->stream);
 }
 
-// Whether multi-step calls advance two steps per launch.
-bool fuses(const lbm_t *h) {
+// Whether multi-step calls may advance two steps per launch.
+bool may_fuse(const lbm_t *h) {
   if (h->kernel != LBM_KERNEL_X2 || onsite(h) || h->fuse == LBM_FUSE_OFF) return false;
   return h->fuse == LBM_FUSE_ALWAYS ||
-         lbm::step2_wins(h->storage, (h->flags & LBM_FORCE) != 0, h->nx, h->ny, h->nz);
+         lbm::step2_sized(h->storage, (h->flags & LBM_FORCE) != 0, h->nx, h->ny, h->nz);
+}
+
+// Whether they do (after ensure_plan2).
+bool fuses(const lbm_t *h, bool moments = false) {
+  const lbm::Step2Plan &p = h->plan2[moments];
+  return may_fuse(h) && p.w != 0 &&
+         (h->fuse == LBM_FUSE_ALWAYS ||
+          lbm::step2_wins(h->storage, (h->flags & LBM_FORCE) != 0,
+                          (h->flags & (LBM_WALL_X | LBM_WALL_Y | LBM_WALL_Z)) != 0, h->pitch,
+                          h->ny, h->nz, p));
 }
 
 // The two-step kernel's tiles, made before the first launch that needs them.
 int ensure_plan2(lbm_t *h, bool moments) {
   lbm::Step2Plan &p = h->plan2[moments];
-  if (p.w != 0 || !fuses(h)) return LBM_OK;
+  if (p.w != 0 || !may_fuse(h)) return LBM_OK;
   LBM_CUDA(lbm::prepare_step2(h->storage, make_args(h, nullptr, nullptr), moments),
            "two-step kernel setup");
   p = lbm::step2_plan(h->storage, (h->flags & LBM_FORCE) != 0, moments, h->nx, h->ny, h->nz,
@@ -675,7 +685,7 @@ int lbm_advance(lbm_t *h, int n, const void *f_in, void *f_out, void *f_tmp, flo
     if (!rho[k] || !u[k]) return fail(LBM_EINVAL, "NULL rho or u buffer");
   if (!rho || h->storage == lbm::kF32) rc = ensure_plan2(h, rho != nullptr);
   if (rc) return rc;
-  const int pairs = fuses(h) && (!rho || h->storage == lbm::kF32) ? n / 2 : 0;
+  const int pairs = fuses(h, rho != nullptr) && (!rho || h->storage == lbm::kF32) ? n / 2 : 0;
   int left = pairs + (n - 2 * pairs);  // passes; they alternate and end in f_out
   const void *in = f_in;
   for (int k = 0; k < n; --left) {

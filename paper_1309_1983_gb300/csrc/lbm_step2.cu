@@ -225,17 +225,32 @@ cudaError_t launch_step2_mom(const StepArgs &a, const Moments2 &m, const Step2Pl
 }
 
 // Where two steps per launch are faster than two launches of the two-node
-// kernel. FP32: from where the lattice outgrows L2 (measured cavity, two
-// launches against one, us a step: 96^3 18.2 / 15.7, 78 x 237 x 27 10.1 / 9.7,
-// 72^3 7.3 / 10.2, 101 x 67 x 45 6.6 / 8.7; with a body force 96^3 28.1 / 22.2,
-// 101 x 67 x 85 17.1 / 16.3). 16-bit storage: only on short rows that start at
-// any offset, which the two-node kernel's loads suit least (FP16 cavity,
-// 45 x 234 x 328 71.2 / 58.5, 86 x 194 x 115 39.1 / 34.8; 160^3 55.6 / 69.3,
-// 78 x 237 x 27 7.5 / 10.0, 193 x 160 x 129 67.1 / 70.4).
-bool step2_wins(int storage, bool force, int nx, int ny, int nz) {
+// kernel. By size: FP32 from where the lattice outgrows L2 (cavity, two launches
+// / one, us a step: 96^3 18.6 / 15.9, 72^3 7.3 / 10.2, 101 x 67 x 45 6.6 / 8.7;
+// with a body force 96^3 24.2 / 22.1); 16-bit storage only on short rows that
+// start at any offset, which the two-node kernel's loads suit least (160^3 55.6 /
+// 69.3, 193 x 160 x 129 67.1 / 70.4).
+bool step2_sized(int storage, bool force, int nx, int ny, int nz) {
   const double nodes = (double)nx * ny * nz;
   if (storage == kF32) return nodes >= (force ? 6e5 : 5e5);
   return nx <= 90 && nx % 16 != 0 && nodes >= 1.5e6;
+}
+
+// And by shape: the rim and the three extra planes of a run cost thin lattices
+// more than the pass saves. The two-node kernel moves 46 padded FP32 nodes per
+// ns; the plan's modelled time has to be shorter than its by a factor that
+// covers what the model leaves out, the collisions above all. Measured, modelled
+// gain: measured gain of one launch. FP32: 1000^2 x 1 0.37: 0.49, 400^2 x 6 0.96:
+// 0.96, 78 x 237 x 27 1.00: 1.07 periodic, 0.92 cavity, 1000 x 3 x 300 1.03: 0.90,
+// 400 x 2 x 2000 1.08: 1.22, 96^3 1.17: 1.22; with a force 256 x 256 x 16 1.08: 0.91,
+// 96^3 1.14: 1.00 to 1.10. FP16 periodic 77 x 3 x 9000 1.60: 0.83, 40 x 5000 x 8 2.01:
+// 0.98, 77 x 300 x 100 2.24: 1.11; FP16 cavity 45 x 200^2 2.36: 0.97, 10 x 500 x 400
+// 2.67: 1.26, 23 x 300^2 2.98: 1.19.
+bool step2_wins(int storage, bool force, bool walls, int pitch, int ny, int nz,
+                const Step2Plan &p) {
+  const double two = 2.0 * pitch * ny * nz / 46e3;
+  const double gain = storage != kF32 ? (walls ? 2.55 : 2.1) : force ? 1.12 : 1.05;
+  return p.us * gain < two;
 }
 
 }  // namespace lbm
