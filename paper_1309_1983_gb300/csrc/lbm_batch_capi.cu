@@ -7,10 +7,8 @@
 #include <string.h>
 
 #include <algorithm>
-#include <functional>
 #include <map>
 #include <new>
-#include <queue>
 #include <tuple>
 #include <vector>
 
@@ -205,9 +203,7 @@ bool pairs_win(const lbm_batch *b) {
 // The items of a two-step pass. Each domain's columns are cut into its best
 // tiles, and the planes of all of them into runs of at most `most`; the value
 // of `most` is the one for which blocks that take the items in order, longest
-// run first, end soonest (a run walks 3 planes more than it writes). More than
-// 6 items per SM were never better (1 to 256 domains of 16 to 96 nodes a side) and
-// cost the first call most: 64 of them 350 us up to 16 an SM, 40 up to 6. False if
+// run first, end soonest (a run walks 3 planes more than it writes). False if
 // they cannot be had (no memory): the calls then go on one step at a time.
 bool upload_items(lbm_batch *b) try {
   if (b->d_items) return true;
@@ -229,6 +225,7 @@ bool upload_items(lbm_batch *b) try {
     if (b->doms[d].nz > deepest) deepest = b->doms[d].nz;
   }
   std::vector<Cut> best;
+  std::vector<double> busy(sms);
   double best_us = 0.0;
   for (int most = deepest; most >= 1; most = most > 4 ? most * 4 / 5 : most - 1) {
     std::vector<Cut> cuts;
@@ -239,21 +236,26 @@ bool upload_items(lbm_batch *b) try {
       cuts.push_back({d, tw[d], th[d], c, tus[d] * ((D.nz + c - 1) / c + 3)});
       n += (size_t)c * ((D.nx + tw[d] - 1) / tw[d]) * ((D.ny + th[d] - 1) / th[d]);
     }
-    if (n > 6 * (size_t)sms && !best.empty()) break;
+    if (n > 16 * (size_t)sms && !best.empty()) break;
     std::stable_sort(cuts.begin(), cuts.end(),
                      [](const Cut &x, const Cut &y) { return x.us > y.us; });
-    std::priority_queue<double, std::vector<double>, std::greater<double>> busy;
-    for (int k = 0; k < sms; ++k) busy.push(0.0);
+    // when each SM is free, as a heap with the soonest first
+    std::fill(busy.begin(), busy.end(), 0.0);
     double end = 0.0;
     for (const Cut &c : cuts) {
       const BatchDom &D = b->doms[c.dom];
       const long long items =
           (long long)c.chunks * ((D.nx + c.w - 1) / c.w) * ((D.ny + c.h - 1) / c.h);
       for (long long k = 0; k < items; ++k) {
-        const double t = busy.top() + c.us;
-        busy.pop();
-        busy.push(t);
+        const double t = busy[0] + c.us;
         if (t > end) end = t;
+        size_t at = 0;
+        for (size_t kid; (kid = 2 * at + 1) < busy.size(); at = kid) {
+          if (kid + 1 < busy.size() && busy[kid + 1] < busy[kid]) ++kid;
+          if (busy[kid] >= t) break;
+          busy[at] = busy[kid];
+        }
+        busy[at] = t;
       }
     }
     if (best.empty() || end < best_us) {
