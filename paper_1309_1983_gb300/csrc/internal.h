@@ -77,9 +77,10 @@ struct Step2Plan {
   float us;  // modelled time of a pass
 };
 // Whether multi-step calls of this lattice are faster so: by its size alone
-// (where no plan is needed to say no), and with the plan.
+// (where no plan is needed to say no), and with the plan (slim: made for a
+// body force or moments).
 bool step2_sized(int storage, bool force, int nx, int ny, int nz);
-bool step2_wins(int storage, bool force, bool walls, int pitch, int ny, int nz,
+bool step2_wins(int storage, bool slim, bool walls, int pitch, int ny, int nz,
                 const Step2Plan &p);
 // Once per handle and device before its launches.
 cudaError_t prepare_step2(int storage, const StepArgs &a, bool moments);

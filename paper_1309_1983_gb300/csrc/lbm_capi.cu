@@ -193,7 +193,7 @@ bool fuses(const lbm_t *h, bool moments = false) {
   const lbm::Step2Plan &p = h->plan2[moments];
   return may_fuse(h) && p.w != 0 &&
          (h->fuse == LBM_FUSE_ALWAYS ||
-          lbm::step2_wins(h->storage, (h->flags & LBM_FORCE) != 0,
+          lbm::step2_wins(h->storage, moments || (h->flags & LBM_FORCE) != 0,
                           (h->flags & (LBM_WALL_X | LBM_WALL_Y | LBM_WALL_Z)) != 0, h->pitch,
                           h->ny, h->nz, p));
 }

@@ -93,6 +93,15 @@ static double step2_plane_us(int bytes, int w, int h) {
   return std::max(0.1 + kb / 48.0, 0.9);
 }
 
+// The same for a lattice's slim block (body force, moments), where the
+// collisions' instructions count as well: 1.4 us for 32 x 7 tiles, 1.9 for
+// 32 x 11. With the traffic alone the plans took tiles too small: FP32 cavity
+// with a force, us a step, 96^3 22.0 / 19.5, 128^3 53.0 / 47.9, 192^3 156.8 / 138.7;
+// with moments too 24.0 / 21.7, 57.6 / 52.5, 168.2 / 153.6 (110^3 32.2 / 33.5).
+static double slim_plane_us(int w, int h) {
+  return std::max(step2_plane_us(4, w, h), 1.0 + 0.0008 * (w + 2) * (h + 2));
+}
+
 // Rows of the rim per thread that a tile of width w may have.
 template <class Block>
 static int step2_rows(int w) {
@@ -129,7 +138,8 @@ static Step2Plan plan_for(int storage, int nx, int ny, int nz, int sms) {
     const int w = w8 < nx ? w8 : nx;
     for (int h = std::min(2 * step2_rows<Block>(w) - 2, ny); h >= 1; --h) {
       const int ntx = (nx + w - 1) / w, nty = (ny + h - 1) / h;
-      const double plane_us = step2_plane_us(bytes, w, h);
+      const double plane_us = std::is_same<Block, SlimBlock>::value
+                                  ? slim_plane_us(w, h) : step2_plane_us(bytes, w, h);
       const long long tiles = (long long)ntx * nty;
       for (int k = 0; k <= 16; ++k) {  // chunks that fill k waves of blocks
         const int c = k == 0 ? 1 : (int)std::min<long long>(nz, (long long)k * sms / tiles);
@@ -242,14 +252,14 @@ bool step2_sized(int storage, bool force, int nx, int ny, int nz) {
 // covers what the model leaves out, the collisions above all. Measured, modelled
 // gain: measured gain of one launch. FP32: 1000^2 x 1 0.37: 0.49, 400^2 x 6 0.96:
 // 0.96, 78 x 237 x 27 1.00: 1.07 periodic, 0.92 cavity, 1000 x 3 x 300 1.03: 0.90,
-// 400 x 2 x 2000 1.08: 1.22, 96^3 1.17: 1.22; with a force 256 x 256 x 16 1.08: 0.91,
-// 96^3 1.14: 1.00 to 1.10. FP16 periodic 77 x 3 x 9000 1.60: 0.83, 40 x 5000 x 8 2.01:
+// 400 x 2 x 2000 1.08: 1.22, 96^3 1.17: 1.22; with a force 101 x 67 x 85 0.92: 0.97,
+// 256 x 256 x 16 0.95: 0.99, 99^3 1.00: 1.14, 96^3 1.12: 1.11. FP16 periodic 77 x 3 x 9000 1.60: 0.83, 40 x 5000 x 8 2.01:
 // 0.98, 77 x 300 x 100 2.24: 1.11; FP16 cavity 45 x 200^2 2.36: 0.97, 10 x 500 x 400
 // 2.67: 1.26, 23 x 300^2 2.98: 1.19.
-bool step2_wins(int storage, bool force, bool walls, int pitch, int ny, int nz,
+bool step2_wins(int storage, bool slim, bool walls, int pitch, int ny, int nz,
                 const Step2Plan &p) {
   const double two = 2.0 * pitch * ny * nz / 46e3;
-  const double gain = storage != kF32 ? (walls ? 2.55 : 2.1) : force ? 1.12 : 1.05;
+  const double gain = storage != kF32 ? (walls ? 2.55 : 2.1) : slim ? 0.99 : 1.05;
   return p.us * gain < two;
 }
 
