@@ -86,7 +86,8 @@ def measured_hbm():
 
 KERNEL_SOURCES = ("paper_1309_1983_gb300/csrc/lbm_step_x2.cu", "paper_1309_1983_gb300/csrc/d3q19.cuh",
                   "paper_1309_1983_gb300/csrc/stream.cuh", "paper_1309_1983_gb300/csrc/internal.h",
-                  "paper_1309_1983_gb300/csrc/pack.cuh", "paper_1309_1983_gb300/csrc/check.cuh")
+                  "paper_1309_1983_gb300/csrc/pack.cuh", "paper_1309_1983_gb300/csrc/check.cuh",
+                  "paper_1309_1983_gb300/csrc/launch.cuh")
 
 
 def code_only(text):
@@ -641,7 +642,8 @@ def run_ours(args):
         L = Lattice(n, n, n, TAU, storage=args.storage)
     u0 = torch.from_numpy(W.shear_wave(n, n, n, AMP)).float().cuda()
     L.init_equilibrium(u=u0 if args.geometry == "periodic" else None)
-    L.step(max(args.warmup, 3))
+    for _ in range(max(args.warmup, 3)):
+        L.step(1)  # the timed calls: a longer call takes two steps per launch
     torch.cuda.synchronize()
 
     props = torch.cuda.get_device_properties(local)

@@ -7,7 +7,8 @@ restores device memory around its passes, ends in about a minute.
 
     python -m paper_1309_1983_gb300.profile_cases step --geometry cavity --storage f16 --n 256
         init + 4 plain step launches (k_step_x2 by default; --kernel x4 / node;
-        --onsite: on-site velocity walls instead of halfway bounce-back)
+        --onsite: on-site velocity walls instead of halfway bounce-back;
+        --per-call 4: calls of four steps, two launches of k_step2 each)
     python -m paper_1309_1983_gb300.profile_cases batch-adjoint --steps 4
         the 64-cavity batch: one forward sequence with moments, then two
         reverse-sequence launches (k_batch_adj_seq) of `steps` steps each
@@ -21,19 +22,20 @@ import sys
 
 
 def step(geometry: str = "cavity", storage: str = "f16", n: int = 256, launches: int = 4,
-         tau: float = 0.55, kernel: str = "x2", onsite: bool = False, rows: int = 0) -> None:
+         tau: float = 0.55, kernel: str = "x2", onsite: bool = False, rows: int = 0,
+         per_call: int = 1, force: bool = False) -> None:
     import torch
     from .lattice import Lattice
     walls = (geometry == "cavity",) * 3
     L = Lattice(n, n, n, tau, walls=walls, lid=(0.05, 0.0, 0.0) if geometry == "cavity" else None,
-                storage=storage, onsite=onsite)
+                storage=storage, onsite=onsite, force=force)
     L.set_graph_steps(0)
     L.set_kernel(kernel)
     if rows:
         L.set_pair_block(32, rows)
     L.init_equilibrium()
     for _ in range(launches):
-        L.step(1)
+        L.step(per_call)
     torch.cuda.synchronize()
     L.close()
 
@@ -75,6 +77,9 @@ def main(argv=None) -> int:
     s.add_argument("--storage", default="f16", choices=["f32", "f16", "bf16"])
     s.add_argument("--n", type=int, default=256)
     s.add_argument("--launches", type=int, default=4)
+    s.add_argument("--per-call", type=int, default=1,
+                   help="steps per call: 4 for two launches of two steps each (k_step2)")
+    s.add_argument("--force", action="store_true", help="with a body force field")
     s.add_argument("--kernel", default="x2", choices=["x2", "x4", "node", "tma"])
     s.add_argument("--rows", type=int, default=0,
                    help="tile rows of the tma kernel (pair-block rows; 0: the default)")
@@ -86,7 +91,7 @@ def main(argv=None) -> int:
     a = p.parse_args(argv)
     if a.case == "step":
         step(a.geometry, a.storage, a.n, a.launches, tau=a.tau, kernel=a.kernel, onsite=a.onsite,
-             rows=a.rows)
+             rows=a.rows, per_call=a.per_call, force=a.force)
     else:
         batch_adjoint(a.steps, a.launches)
     print("ok")
