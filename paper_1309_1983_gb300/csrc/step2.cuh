@@ -447,7 +447,7 @@ __device__ __forceinline__ void step2_second(const typename Store<S>::T *__restr
   P2 Fnext[3] = {};
   if constexpr (FORCE) force(za, Fnext);
 
-  const int pad = Dom::kPadded && x0 + cw == D.nx ? D.pitch - D.nx : 0;
+  [[maybe_unused]] const int pad = x0 + cw == D.nx ? D.pitch - D.nx : 0;  // after its rows
 
   // plane za - 1 + j of the first step is in slots j modulo (4, 3, 2 or 3);
   // the output plane za - 1 + j pulls from j - 1, j and j + 1
@@ -509,13 +509,16 @@ __device__ __forceinline__ void step2_second(const typename Store<S>::T *__restr
         if (b_live) Store<S>::st(D.template dst<i>(zoff + ob, ps), v.y);
       });
     }
-    for (int j = t; j < pad * ch; j += THREADS) {
-      const uint32_t ps = D.stride();
-      const uint32_t off = (uint32_t)z * row + (uint32_t)(y0 + j / pad) * D.pitch + D.nx + j % pad;
-      static_for<0, Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        Store<S>::st(D.template dst<i>(off, ps), 0.0f);
-      });
+    if constexpr (Dom::kPadded) {
+      for (int j = t; j < pad * ch; j += THREADS) {
+        const uint32_t ps = D.stride();
+        const uint32_t off =
+            (uint32_t)z * row + (uint32_t)(y0 + j / pad) * D.pitch + D.nx + j % pad;
+        static_for<0, Q>([&](auto I) {
+          constexpr int i = decltype(I)::value;
+          Store<S>::st(D.template dst<i>(off, ps), 0.0f);
+        });
+      }
     }
     if (z + 1 < zb) __syncthreads();
     sp = (sp + 1) & 3;
