@@ -193,8 +193,8 @@ int upload_tables(lbm_batch *b) {
 // Whether two steps per launch beat the persistent launch, both modelled per
 // step from measurements: 3.2 us a barrier and 46 nodes per ns against 1.12
 // times the items' time and half a launch. Measured old / new, us a step:
-// 64 cavities of 16..96 (11.4 M nodes) 270 / 224, 16 of them 63.2 / 55.0, 8
-// 22.2 / 22.0, 4 (0.29 M) 9.4 / 11.3, 1 (0.05 M) 5.5 / 4.0.
+// 64 cavities of 16..96 (11.4 M nodes) 270 / 217, 16 of them 63.2 / 55.0, 8
+// 22.2 / 20.3, 4 (0.29 M) 9.4 / 11.3, 1 (0.05 M) 5.5 / 3.8.
 bool pairs_win(const lbm_batch *b) {
   if (b->fuse != LBM_FUSE_AUTO) return b->fuse == LBM_FUSE_ALWAYS;
   return 0.56 * b->pass_us + 0.5 < 3.2 + (double)b->cells / 46e3;
@@ -972,6 +972,12 @@ int lbm_batch_autotune(lbm_batch_t *b, const char *cache_path, int steps, int *t
   }
   // tile sizes x resident blocks per SM (0 = as many as fit) of the
   // persistent launch; the untimed first call also captures its graph
+  struct KeepFuse {  // the tiling is that of the persistent launch
+    lbm_batch_t *b;
+    int fuse;
+    ~KeepFuse() { b->fuse = fuse; }
+  } keep{b, b->fuse};
+  b->fuse = LBM_FUSE_OFF;
   static const int kThreads[] = {64, 128, 256};
   static const int kBps[] = {0, 2, 4, 6, 8};
   int best_t = 0, best_b = 0;
