@@ -222,10 +222,11 @@ int lbm_set_kernel(lbm_t *h, int variant);
  * result is in the same buffer as after single steps. The other steps and
  * steps that write rho and u take one launch each. Results are identical.
  * After such a call the other buffer of the pair holds an earlier state, not
- * always the one before the last step. LBM_FUSE_AUTO (default): for the
- * lattices that it is faster for (FP32 from 500,000 nodes on, 600,000 with a body force, and
- * large 16-bit lattices of short rows);
- * LBM_FUSE_OFF: never; LBM_FUSE_ALWAYS: whenever the kernel and the walls
+ * always the one before the last step, and row padding holds zeros.
+ * LBM_FUSE_AUTO (default): for the
+ * lattices that it is faster for (FP32 from 500,000 nodes on, 600,000 with a
+ * body force, and large 16-bit lattices of short rows, unless they are thin
+ * along an axis); LBM_FUSE_OFF: never; LBM_FUSE_ALWAYS: whenever the kernel and the walls
  * allow it. Returns LBM_EINVAL for any other mode. */
 #define LBM_FUSE_AUTO 0
 #define LBM_FUSE_OFF 1

@@ -8,8 +8,8 @@ lbm_adjoint_u0, or their lbm_batch_* counterparts for a batch of lattices).
 The forward keeps the states f^0, f^K, f^2K, ...; the backward recomputes
 each segment from its checkpoint and then runs the reverse steps over it.
 By default (``moments=True``) the recompute stores, per step, only the
-density and velocity its collision used (16 bytes per node): the collision Jacobian depends on the pulled state only through
-them, so the reverse step (lbm_adjoint_step_moments) reads those instead of
+density and velocity its collision used (16 bytes per node): the collision
+Jacobian depends on the pulled state only through them, so the reverse step (lbm_adjoint_step_moments) reads those instead of
 re-gathering f^n, and a segment needs 16 instead of 76 bytes per node and
 step. ``moments=False`` keeps the K - 1 segment states and re-gathers them
 (lbm_adjoint_step); both give the same bits.
@@ -196,6 +196,7 @@ class AdjointProblem(_Checkpointed):
 
     @property
     def launches_forward(self):
+        """At one step per launch; large lattices take two (lbm_set_fusion)."""
         return 1 + self.T
 
     def _fbuf(self):

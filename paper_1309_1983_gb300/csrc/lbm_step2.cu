@@ -7,16 +7,20 @@
 // (7 TB/s: a tile also reads its rim, 190 bytes per node and pass for 32 x 14
 // tiles against 152) and, at 86% of the DRAM rate of a copy, nearly DRAM.
 // Measured on GB300, MLUPS x 1e-3, one step per launch against two:
-//   periodic FP32   128^3 43.6 / 58.7   256^3 46.0 / 72.4   384^3 46.6 / 68.8
-//   cavity FP32     128^3 43.8 / 55.4   256^3 46.1 / 60.0   384^3 46.6 / 61.2
-//   cavity FP32     23 x 374 x 236 28.5 / 44.5   273 x 213 x 113 42.1 / 53.3
-//   periodic FP16   384^3 83.7 / 75.7   45 x 234 x 328 48.1 / 66.4
+//   periodic FP32   128^3 43.7 / 59.6   256^3 46.0 / 72.9   384^3 46.6 / 69.1
+//   cavity FP32     128^3 43.9 / 55.4   256^3 46.2 / 63.6   384^3 46.7 / 64.4
+//   cavity FP32     45 x 234 x 328 31.7 / 55.9   273 x 213 x 113 41.9 / 55.3
+//   with a force    128^3 40.9 / 47.5   128^3 cavity 38.7 / 43.9
+//   periodic FP16   384^3 83.7 / 74.7   45 x 234 x 328 52.3 / 68.4
 // 16-bit storage moves half the bytes, so there the two collisions and the
-// conversions bound the pass.
+// conversions bound the pass. Counters at 256^3 periodic FP32: 77.5 bytes read and
+// 72.8 written per node and pass, 5.5 TB/s of DRAM, issue 40%; of 9.5 stalled
+// cycles per instruction 3.0 at the barrier and 2.1 on loads, so latency is what
+// is left, and 16 warps of 128 registers are all that fit.
 //
 // One block per SM of 9 + 7 warps at 128 registers (7 + 5 at 168 with a body
-// force or moments, which spill at 128: 256^3 periodic with both 435 / 340 us
-// a step). Tried and slower, 384^3
+// force or moments, which spill at 128: 128^3 periodic with both 90.6 us a step
+// there, 48.2 here). Tried and slower, 384^3
 // periodic FP32: all warps alternating between the two steps with a barrier
 // after each (48.6 without, 65.3 with the next plane's loads in flight over
 // the second step), 11 + 9 warps at 96 registers (59.9, spills), 7 + 5 at
@@ -33,9 +37,8 @@
 
 namespace lbm {
 
-// Body force and moments need more registers than the wide block has (128^3
-// with both 90.6 us a step there, 52.8 in the slim one; without either 35.7
-// and 42.6).
+// Body force and moments need more registers than the wide block has; without
+// either it is the faster one (128^3 periodic 35.2 us a step, 42.6 in the slim).
 template <bool FORCE, bool MOM>
 using BlockOf = std::conditional_t<FORCE || MOM, SlimBlock, WideBlock>;
 
