@@ -191,3 +191,28 @@ def test_batch_advance_with_and_without_moments(walls):
     for fields in (0, B.cells):
         _against_singles("lbm_batch_advance", B.handle, B.current_buffers()[0], fields,
                          B.set_fusion)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("geom", ["periodic", "cavity"])
+@pytest.mark.parametrize("shape", [(37, 6, 5), (20, 33, 4), (1, 9, 3), (131, 5, 7)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_writes_nodes_and_zeros_in_the_padding(shape, geom, storage):
+    """Nothing behind the buffers changes, and row padding ends as zeros."""
+    from paper_1309_1983_gb300.lattice import Lattice
+    nx, ny, nz = shape
+    walls, lid = GEOMS[geom]
+    L = Lattice(nx, ny, nz, 0.7, walls=tuple(bool(w) for w in walls), lid=lid, storage=storage)
+    nb, eb, pitch = L.layout.f_bytes, L.layout.elem_bytes, L.layout.pitch
+    full = [torch.full((nb + 4096,), 0xFF, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    L.f_a, L.f_b = full[0][:nb], full[1][:nb]
+    L._bind()
+    L.set_fusion("always")
+    L.init_equilibrium()
+    L.step(4)
+    torch.cuda.synchronize()
+    for b in full:
+        assert bool((b[nb:] == 0xFF).all())
+        rows = b[:19 * nz * ny * pitch * eb].view(19, nz, ny, pitch * eb)
+        assert bool((rows[..., nx * eb:] == 0).all())
+    L.close()
